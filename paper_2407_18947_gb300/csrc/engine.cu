@@ -1163,6 +1163,26 @@ ContractPlan& Engine<R>::plan(const std::string& spec, const View& A, const View
   P->a_off0 = h[iaB];
   P->b_off0 = h[ibB];
   P->c_off0 = h[icB];
+  P->c_unit_m = !gm.empty() && std::llabs(gm.back().sc) == 1;
+  // FP64 products above a few million multiply-adds: sliced products on the
+  // tensor cores (oz_gemm.h).  Both sides in SM clocks: the CUDA cores do two
+  // FP64 multiply-adds per SM and clock (four per complex one, 85 % of that
+  // rate at best), the sliced form costs what its plan estimates.  Measured,
+  // CUDA cores against sliced: 3800 x 14440 x 48 17.6 -> 2.17 ms, 3800 x 38 x
+  // 14440 24.5 -> 1.79 ms, 451 x 451 x 451 0.87 -> 0.09 ms; on the other side
+  // of the line 10 x 10 x 5.5e6 (4.3 against 8.5 ms) and 144400 x 1 x 380
+  // (0.42 against 0.67 ms) stay on the CUDA cores.
+  if (std::is_same<R, double>::value && NB == 1 && K >= 8) {
+    const OzPlan oz = oz_plan(M, N, K);
+    const double simt = 4.0 * double(M) * double(N) * double(K) / (2.0 * 152.0 * 0.85) + 4000.0;
+    if (simt > oz.cost) {
+      P->use_oz = true;
+      P->oz = oz;
+      ContractPlan& ref = *P;
+      plans_[key] = std::move(P);
+      return ref;
+    }
+  }
   // small outputs (held whole by every CTA, K split over the GPU) and single
   // long output columns get their own kernels
   {
@@ -1321,6 +1341,10 @@ void Engine<R>::run_contract(const std::string& spec, double alpha, const View& 
   pc += sc;
   if (P.use_tc) {
     run_contract_tc(P, alpha, pa, pb, pc, accumulate);
+    return;
+  }
+  if (P.use_oz) {
+    run_contract_oz(P, alpha, pa, pb, pc, accumulate);
     return;
   }
   if (P.kind != 0) {
@@ -1488,6 +1512,31 @@ void Engine<R>::run_contract_tc(ContractPlan& P, double alpha, const C* pa, cons
   } else {
     (void)P; (void)alpha; (void)pa; (void)pb; (void)pc; (void)accumulate;
     throw Error(kErrState, "tensor-core route requires a complex64 graph");
+  }
+}
+
+template <typename R>
+void Engine<R>::run_contract_oz(ContractPlan& P, double alpha, const C* pa, const C* pb, C* pc,
+                                bool accumulate) {
+  if constexpr (std::is_same<R, double>::value) {
+    const bool sw = P.oz.swap;
+    const OzOperand a{pa, P.a_off0, P.aM, P.aK, P.a_kcontig}, b{pb, P.b_off0, P.bN, P.bK, P.b_kcontig};
+    const int Mg = sw ? P.N : P.M, Ng = sw ? P.M : P.N;
+    C* part = nullptr;
+    if (P.oz.nsplit > 1)
+      part = static_cast<C*>(scratch(split_slot_, size_t(P.oz.nsplit) * P.M * P.N * sizeof(C)));
+    int* err = error_flag();
+    const int pk = pbegin();
+    launches_ += oz_gemm(P.oz, sw ? b : a, sw ? a : b, Mg, Ng, P.K, pc, P.c_off0, sw ? P.cN : P.cM,
+                         sw ? P.cM : P.cN, P.c_unit_m != sw, alpha, accumulate, part, err,
+                         wait_budget_, stream_);
+    const double mnk = double(P.M) * P.N * P.K;
+    pend(pk, "contract_sliced_c128", 8.0 * mnk,
+         (double(P.M) * P.K + double(P.N) * P.K + double(P.M) * P.N * (accumulate ? 2.0 : 1.0)) * sizeof(C),
+         cur_detail_);
+  } else {
+    (void)P; (void)alpha; (void)pa; (void)pb; (void)pc; (void)accumulate;
+    throw Error(kErrState, "the sliced route requires a complex128 graph");
   }
 }
 

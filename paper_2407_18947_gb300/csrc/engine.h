@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "common.h"
+#include "oz_gemm.h"
 
 namespace rtcc3 {
 
@@ -68,6 +69,10 @@ struct ContractPlan {
   bool use_tc = false, tc_swap = false;
   int tc_nsplit = 1, tc_kp = 0;
   bool tc_out = false;  // short sum bound by its output (two CTAs per SM)
+  // FP64 products large enough for the sliced tensor-core form
+  bool use_oz = false;
+  bool c_unit_m = false;  // C's contiguous index is on the M side
+  OzPlan oz;
   long long a_off0 = 0, b_off0 = 0, c_off0 = 0;  // batch-0 offsets (host copies)
   long long *aM = nullptr, *aK = nullptr, *bN = nullptr, *bK = nullptr;
   long long *cM = nullptr, *cN = nullptr, *aB = nullptr, *bB = nullptr, *cB = nullptr;
@@ -442,6 +447,8 @@ class Engine {
   void run_contract_small(ContractPlan& P, double alpha, const C* pa, const C* pb, C* pc,
                           bool accumulate);
   void run_contract_tc(ContractPlan& P, double alpha, const C* pa, const C* pb, C* pc,
+                       bool accumulate);
+  void run_contract_oz(ContractPlan& P, double alpha, const C* pa, const C* pb, C* pc,
                        bool accumulate);
   int launches_ = 0;
   int generation_ = 0;

@@ -20,6 +20,7 @@
 // Every mbarrier wait is bounded by a clock budget; on expiry the kernel
 // raises *err and winds down, releasing its tensor memory.
 #include "tc_gemm.h"
+#include "tc_ptx.h"
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -32,52 +33,10 @@ namespace rtcc3 {
 namespace {
 
 constexpr int kBM = 128;
-// Waits on other warps' progress spin for at most a budget of clock cycles
-// (a kernel argument, kWaitBudget by default, about 2 s).  Waits for this
-// CTA's own asynchronous work to land (its TMA / bulk copies, its MMAs) at
-// exit use kDrainBudget: that work completes by itself, so these waits end
-// whatever the progress budget was; they are what makes giving up safe
-// (no copy or MMA may still target the CTA's shared or tensor memory when it
-// frees them).
-constexpr long long kWaitBudget = 4000000000LL;
-constexpr long long kDrainBudget = 4000000000LL;
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long long budget) {
-  const long long t0 = clock64();
-  while (true) {
-    uint32_t ok = 0;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return true;
-    if (clock64() - t0 > budget) return false;
-  }
-}
-
 __device__ __forceinline__ uint32_t to_tf32(float x) {
   uint32_t r;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
   return r;
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-               : "memory");
 }
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y,
@@ -176,12 +135,6 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
       "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]),
       "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]),
       "r"(r[29]), "r"(r[30]), "r"(r[31])
-      : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
       : "memory");
 }
 
