@@ -337,6 +337,7 @@ StageNodes eval_stage(rtcc3_ctx* ctx, int b, const double2* ybase, const double2
     RTCC3_CUDA(cudaMemcpy(&bad, ctx->checkflag, sizeof(int), cudaMemcpyDeviceToHost));
     if (bad) {
       RTCC3_CUDA(cudaMemset(ctx->checkflag, 0, sizeof(int)));
+      RTCC3_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
       throw Error(RTCC3_ERR_STATE, "checked mode: a device tensor was written past its end");
     }
   }
@@ -396,8 +397,8 @@ void setup_runner(rtcc3_ctx* ctx, const double* Lfac) {
               (ctx->eps_h[o + c] - shift);
     H.osum = rn->template alloc<double>(os.size());
     H.vsum = rn->template alloc<double>(vs.size());
-    RTCC3_CUDA(cudaMemcpy(H.osum, os.data(), os.size() * sizeof(double), cudaMemcpyHostToDevice));
-    RTCC3_CUDA(cudaMemcpy(H.vsum, vs.data(), vs.size() * sizeof(double), cudaMemcpyHostToDevice));
+    upload(H.osum, os.data(), os.size() * sizeof(double));
+    upload(H.vsum, vs.data(), vs.size() * sizeof(double));
     // the sums rounded once to the compute precision (the dense triples
     // kernels divide in R; after the mid-gap shift every occupied sum is
     // negative and every virtual sum positive, so D = vsum - osum adds two
@@ -405,8 +406,8 @@ void setup_runner(rtcc3_ctx* ctx, const double* Lfac) {
     std::vector<R> osr(os.begin(), os.end()), vsr(vs.begin(), vs.end());
     H.osum_r = rn->template alloc<R>(osr.size());
     H.vsum_r = rn->template alloc<R>(vsr.size());
-    RTCC3_CUDA(cudaMemcpy(H.osum_r, osr.data(), osr.size() * sizeof(R), cudaMemcpyHostToDevice));
-    RTCC3_CUDA(cudaMemcpy(H.vsum_r, vsr.data(), vsr.size() * sizeof(R), cudaMemcpyHostToDevice));
+    upload(H.osum_r, osr.data(), osr.size() * sizeof(R));
+    upload(H.vsum_r, vsr.data(), vsr.size() * sizeof(R));
     // occupied blocks in orbit order: for each i <= j <= k its distinct
     // permutations, one after the other
     std::vector<int> order;
@@ -423,15 +424,14 @@ void setup_runner(rtcc3_ctx* ctx, const double* Lfac) {
         }
     RTCC3_CHECK(order.size() == size_t(o) * o * o, kErrState, "orbit order incomplete");
     H.orbit_order = rn->template alloc<int>(order.size());
-    RTCC3_CUDA(cudaMemcpy(H.orbit_order, order.data(), order.size() * sizeof(int),
-                          cudaMemcpyHostToDevice));
+    upload(H.orbit_order, order.data(), order.size() * sizeof(int));
   }
   H.h = rn->template alloc<Cx<R>>(hc.size());
   H.L = rn->template alloc<Cx<R>>(Lc.size());
   H.ones = rn->template alloc<Cx<R>>(n);
-  RTCC3_CUDA(cudaMemcpy(H.h, hc.data(), hc.size() * sizeof(Cx<R>), cudaMemcpyHostToDevice));
-  RTCC3_CUDA(cudaMemcpy(H.L, Lc.data(), Lc.size() * sizeof(Cx<R>), cudaMemcpyHostToDevice));
-  RTCC3_CUDA(cudaMemcpy(H.ones, ones.data(), ones.size() * sizeof(Cx<R>), cudaMemcpyHostToDevice));
+  upload(H.h, hc.data(), hc.size() * sizeof(Cx<R>));
+  upload(H.L, Lc.data(), Lc.size() * sizeof(Cx<R>));
+  upload(H.ones, ones.data(), ones.size() * sizeof(Cx<R>));
   rn->E.set_profiler(&ctx->prof);
   rn->E.set_wait_budget(ctx->opt.spin_budget);
   rn->E.set_checked(ctx->opt.checked != 0);
@@ -565,6 +565,7 @@ void check_device_timeout(rtcc3_ctx* ctx) {
   RTCC3_CUDA(cudaMemcpy(&flag, E.error_flag(), sizeof(int), cudaMemcpyDeviceToHost));
   if (flag) {
     RTCC3_CUDA(cudaMemset(E.error_flag(), 0, sizeof(int)));
+    RTCC3_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
     if (flag & kEigStatusBase) {
       const int reason = (flag >> 20) & 0xf, n = (flag >> 10) & 0x3ff, row = flag & 0x3ff;
       throw Error(reason == kEigNonFinite ? RTCC3_ERR_NONFINITE : RTCC3_ERR_TIMEOUT,
@@ -833,7 +834,7 @@ void ground_state_impl(rtcc3_ctx* ctx, double tol, int maxiter) {
   RTCC3_CUDA(cudaStreamSynchronize(ctx->stream));
   ctx->time = 0.0;
   ctx->step_total = 0;
-  RTCC3_CUDA(cudaMemcpy(ctx->tdev, &ctx->time, sizeof(double), cudaMemcpyHostToDevice));
+  upload(ctx->tdev, &ctx->time, sizeof(double));
 }
 
 // Triples-only map (t1, t2) -> (X1, X2) and its vector-Jacobian product.
@@ -1111,8 +1112,8 @@ int rtcc3_create(int nocc, int nvir, int nbatch, const rtcc3_options* opt, rtcc3
     raw->checkflag = raw->dalloc<int>(1);
     RTCC3_CUDA(cudaMemset(raw->checkflag, 0, sizeof(int)));
     raw->fhost.assign(nbatch, FieldDev{0, 0.0, 0.0, 0.0, 1.0, {0.0, 0.0, 1.0}});
-    RTCC3_CUDA(cudaMemcpy(raw->fdev, raw->fhost.data(), nbatch * sizeof(FieldDev), cudaMemcpyHostToDevice));
-    RTCC3_CUDA(cudaMemcpy(raw->fnone, raw->fhost.data(), sizeof(FieldDev), cudaMemcpyHostToDevice));
+    upload(raw->fdev, raw->fhost.data(), nbatch * sizeof(FieldDev));
+    upload(raw->fnone, raw->fhost.data(), sizeof(FieldDev));
     RTCC3_CUDA(cudaMemset(raw->y, 0, raw->ny * nbatch * sizeof(double2)));
     RTCC3_CUDA(cudaMemset(raw->tdev, 0, sizeof(double)));
   });
@@ -1146,8 +1147,8 @@ int rtcc3_set_hamiltonian(rtcc3_ctx* ctx, const double* eps, int naux, const dou
     ctx->mu_h.assign(dipole, dipole + size_t(3) * n * n);
     if (!ctx->eps) ctx->eps = ctx->dalloc<double>(n);
     if (!ctx->mu) ctx->mu = ctx->dalloc<double>(size_t(3) * n * n);
-    RTCC3_CUDA(cudaMemcpy(ctx->eps, eps, n * sizeof(double), cudaMemcpyHostToDevice));
-    RTCC3_CUDA(cudaMemcpy(ctx->mu, dipole, size_t(3) * n * n * sizeof(double), cudaMemcpyHostToDevice));
+    upload(ctx->eps, eps, n * sizeof(double));
+    upload(ctx->mu, dipole, size_t(3) * n * n * sizeof(double));
     drop_graph(ctx);
     ctx->runner.reset();
     if (ctx->fp64()) setup_runner<double>(ctx, Lfac);
@@ -1155,7 +1156,7 @@ int rtcc3_set_hamiltonian(rtcc3_ctx* ctx, const double* eps, int naux, const dou
     RTCC3_CUDA(cudaMemset(ctx->y, 0, ctx->ny * ctx->nb * sizeof(double2)));
     ctx->time = 0.0;
     ctx->step_total = 0;
-    RTCC3_CUDA(cudaMemcpy(ctx->tdev, &ctx->time, sizeof(double), cudaMemcpyHostToDevice));
+    upload(ctx->tdev, &ctx->time, sizeof(double));
     size_t fr = 0, tot = 0;
     RTCC3_CUDA(cudaMemGetInfo(&fr, &tot));
     ctx->free_at_setup = fr;
@@ -1278,7 +1279,7 @@ int rtcc3_set_field(rtcc3_ctx* ctx, int b, int kind, double amplitude, double om
     if (dir) { f.dir[0] = dir[0]; f.dir[1] = dir[1]; f.dir[2] = dir[2]; }
     ctx->fhost[b] = f;
     drop_graph(ctx);  // field parameters live on the device, sweep counts do not
-    RTCC3_CUDA(cudaMemcpy(ctx->fdev + b, &f, sizeof(FieldDev), cudaMemcpyHostToDevice));
+    upload(ctx->fdev + b, &f, sizeof(FieldDev));
   });
 }
 
@@ -1296,7 +1297,7 @@ int rtcc3_set_amplitudes(rtcc3_ctx* ctx, int b, const double* t1, const double* 
       if (!src[k]) continue;
       for (size_t t = 0; t < 2 * cnt[k]; ++t)
         RTCC3_CHECK(std::isfinite(src[k][t]), RTCC3_ERR_ARG, "non-finite amplitude");
-      RTCC3_CUDA(cudaMemcpy(yb + off[k], src[k], cnt[k] * sizeof(double2), cudaMemcpyHostToDevice));
+      upload(yb + off[k], src[k], cnt[k] * sizeof(double2));
     }
   });
 }
@@ -1323,7 +1324,7 @@ int rtcc3_set_time(rtcc3_ctx* ctx, double time) {
   return guarded(ctx, [&] {
     RTCC3_CHECK(std::isfinite(time), RTCC3_ERR_ARG, "non-finite time");
     ctx->time = time;
-    RTCC3_CUDA(cudaMemcpy(ctx->tdev, &time, sizeof(double), cudaMemcpyHostToDevice));
+    upload(ctx->tdev, &time, sizeof(double));
   });
 }
 
@@ -1544,10 +1545,10 @@ int rtcc3_set_state(rtcc3_ctx* ctx, const void* buf, long long bytes) {
     uint64_t h = 0;
     std::memcpy(&h, p + sizeof(hd) + body, sizeof(h));
     RTCC3_CHECK(h == fnv1a(p, sizeof(hd) + body), RTCC3_ERR_ARG, "state image checksum mismatch");
-    RTCC3_CUDA(cudaMemcpy(ctx->y, p + sizeof(hd), body, cudaMemcpyHostToDevice));
+    upload(ctx->y, p + sizeof(hd), body);
     ctx->time = hd.time;
     ctx->step_total = hd.step;
-    RTCC3_CUDA(cudaMemcpy(ctx->tdev, &ctx->time, sizeof(double), cudaMemcpyHostToDevice));
+    upload(ctx->tdev, &ctx->time, sizeof(double));
   });
 }
 
@@ -1595,7 +1596,7 @@ int rtcc3_set_observables(rtcc3_ctx* ctx, int nops, const double* ops) {
     ctx->nobs = 0;
     if (nops > 0) {
       RTCC3_CUDA(cudaMalloc(&ctx->obs_ops, nn * nops * sizeof(double2)));
-      RTCC3_CUDA(cudaMemcpy(ctx->obs_ops, ops, nn * nops * sizeof(double2), cudaMemcpyHostToDevice));
+      upload(ctx->obs_ops, ops, nn * nops * sizeof(double2));
       ctx->nobs = nops;
     }
     drop_graph(ctx);  // the observables kernel's grid depends on nops

@@ -46,6 +46,15 @@ enum Status {
 #define RTCC3_CHECK(cond, code, msg)                                              \
   do { if (!(cond)) throw ::rtcc3::Error((code), (msg)); } while (0)
 
+// Host-to-device copy that has landed when the call returns.  cudaMemcpy from
+// pageable memory may return once the bytes are staged, and the library's
+// streams are non-blocking: a kernel launched right after it could read the
+// destination before the copy does.
+inline void upload(void* dst, const void* src, size_t bytes) {
+  RTCC3_CUDA(cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice));
+  RTCC3_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
+}
+
 // Optional per-kernel timing with CUDA events (eager launches only: CUDA
 // graphs are not used while it is enabled).  Each launch is bracketed by an
 // event pair on the launching stream; collect() synchronises and adds the

@@ -849,6 +849,7 @@ int* Engine<R>::error_flag() {
     } else {
       RTCC3_CUDA(cudaMalloc(&err_, sizeof(int)));
       RTCC3_CUDA(cudaMemset(err_, 0, sizeof(int)));
+      RTCC3_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
     }
   }
   return err_;
@@ -1155,7 +1156,7 @@ ContractPlan& Engine<R>::plan(const std::string& spec, const View& A, const View
                                cudaMemcpyHostToDevice, stream_));
   } else {
     RTCC3_CUDA(cudaMalloc(&P->dev, h.size() * sizeof(long long)));
-    RTCC3_CUDA(cudaMemcpy(P->dev, h.data(), h.size() * sizeof(long long), cudaMemcpyHostToDevice));
+    upload(P->dev, h.data(), h.size() * sizeof(long long));
   }
   long long* d = static_cast<long long*>(P->dev);
   P->aM = d + iaM; P->aK = d + iaK; P->bN = d + ibN; P->bK = d + ibK;
