@@ -57,12 +57,12 @@ struct Runner : Base {
       bb.Mo = alloc<double2>(oo);
       bb.So = alloc<double2>(oo);
       bb.Sio = alloc<double2>(oo);
-      bb.wso = alloc<double2>(3 * oo);
+      bb.wso = alloc<double2>(eig_ws(o));
       bb.lo = alloc<double2>(o);
       bb.Mv = alloc<double2>(vv);
       bb.Sv = alloc<double2>(vv);
       bb.Siv = alloc<double2>(vv);
-      bb.wsv = alloc<double2>(3 * vv);
+      bb.wsv = alloc<double2>(eig_ws(v));
       bb.lv = alloc<double2>(v);
     }
     return &bb;
@@ -260,7 +260,7 @@ void launch_basis_ahead(rtcc3_ctx* ctx, const BasisBuffers& bb, const double2* b
   const EigJob jv{bb.Mv, ctx->v, bb.Sv, bb.Siv, bb.lv, bb.wsv, E.eig_sweep_cap()};
   launch_eig(jo, jv, sizeof(R) == 4, E.error_flag(), ss);
   E.prof_end(pk, ss, "field_eig_ahead", 0.0, 0.0);
-  E.add_launches(2);
+  E.add_launches(3);
 }
 
 // Slab size of the blocked triples for this context (0: stored whole).

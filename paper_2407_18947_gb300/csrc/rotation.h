@@ -27,7 +27,7 @@ __host__ __device__ constexpr int eig_status(int reason, int n, int row) {
 }
 
 // One matrix M[n][n] (row-major, complex128) -> S, S^-1 (row-major, complex128)
-// and eigenvalues lam[n]; ws holds 3 n^2 complex128 of scratch.
+// and eigenvalues lam[n]; ws holds eig_ws(n) complex128 of scratch.
 struct EigJob {
   const double2* M;
   int n;
@@ -35,16 +35,23 @@ struct EigJob {
   double2* Sinv;
   double2* lam;
   double2* ws;
-  int max_sweeps = 0;  // QR sweeps before giving up (0: 60 n + 100)
+  int max_sweeps = 0;  // corrections, then QR sweeps, before giving up (0: 10, 60 n + 100)
 };
-// Both matrices of a stage in one launch (one warp each).  fp32: complex64
-// arithmetic (for the complex64 graphs), else complex128.  *status is raised
-// if the QR sweeps do not converge or a matrix is not finite.
+// Scratch of one matrix in complex128 elements, and the word at its end that
+// says the matrix is done.
+__host__ __device__ constexpr size_t eig_ws(int n) { return 8 * size_t(n) * n + size_t(n) + 16; }
+__host__ __device__ inline int* eig_done(double2* ws, int n) {
+  return reinterpret_cast<int*>(ws + eig_ws(n) - 1);
+}
+// Both matrices of a stage (two launches: the refinement of the identity and,
+// for a matrix it leaves, the QR algorithm).  fp32: complex64 arithmetic (for
+// the complex64 graphs), else complex128.  *status is raised if the QR sweeps
+// do not converge or a matrix is not finite.
 void launch_eig(const EigJob& a, const EigJob& b, bool fp32, int* status, cudaStream_t s);
 
 // The eigenbasis of one stage computed ahead of it (complex128, owned by the
 // caller and kept between stages): M* the matrices, S*, Si* = S^-1, l* the
-// eigenvalues, ws* the eigensolver scratch (3 n^2 each).
+// eigenvalues, ws* the eigensolver scratch (eig_ws(n) each).
 struct BasisBuffers {
   double2 *Mo = nullptr, *Mv = nullptr, *So = nullptr, *Sio = nullptr, *Sv = nullptr,
           *Siv = nullptr, *lo = nullptr, *lv = nullptr, *wso = nullptr, *wsv = nullptr;

@@ -42,8 +42,8 @@ FieldBasis<R> start_field_basis(Engine<R>& E, const Hamil<R>& H, int wt,
   bb.Siv = c2(size_t(v) * v);
   bb.lo = c2(o);
   bb.lv = c2(v);
-  bb.wso = c2(3 * size_t(o) * o);
-  bb.wsv = c2(3 * size_t(v) * v);
+  bb.wso = c2(eig_ws(o));
+  bb.wsv = c2(eig_ws(v));
   if (ahead) bb = *ahead;
   double2 *So64 = bb.So, *Sio64 = bb.Sio, *Sv64 = bb.Sv, *Siv64 = bb.Siv, *lo = bb.lo, *lv = bb.lv;
   FieldBasis<R> B;
@@ -69,7 +69,7 @@ FieldBasis<R> start_field_basis(Engine<R>& E, const Hamil<R>& H, int wt,
   launch_to_precision<R>(Sv64, E.data(B.Sv), size_t(v) * v, ss);
   launch_to_precision<R>(Siv64, E.data(B.Siv), size_t(v) * v, ss);
   E.prof_end(pk, ss, "field_eig", 0.0, 0.0);
-  E.add_launches(ahead ? 5 : 7);
+  E.add_launches(ahead ? 5 : 8);
   return B;
 }
 
