@@ -300,6 +300,121 @@ void launch_cfg(bool a_kc, bool b_kc, const Cx<R>* A, long long aoff, const long
   }
 }
 
+// ---- small products spread over the GPU (FineArgs) ----------------------------
+// The tiled kernels give a 38 x 38 x 38 product to one or a few CTAs, which
+// multiply a zero-padded tile: in FP64 that is 40 to 270 us on an SM with two
+// FP64 lanes per clock, in FP32 ten dependent load-barrier-multiply rounds.
+// Here every lane owns a few terms of one output and all its loads are
+// independent, so a product takes about the latency of one load chain
+// (tables, operands): bound by latency below about 1e5 terms, by the FP64
+// pipe (two terms per SM and 4 clocks) above.
+template <typename R>
+__device__ __forceinline__ void fine_sum(const FineArgs<R>& a, const Cx<R>* pa, const Cx<R>* pb,
+                                         int k, int step, R& sr, R& si) {
+  R r0 = R(0), i0 = R(0), r1 = R(0), i1 = R(0);
+  const bool lin = a.aks >= 0 && a.bks >= 0;
+  auto at = [&](int kk, Cx<R>& x, Cx<R>& y) {
+    x = pa[lin ? kk * a.aks : a.aK[kk]];
+    y = pb[lin ? kk * a.bks : a.bK[kk]];
+  };
+  for (; k + 3 * step < a.K; k += 4 * step) {
+    Cx<R> x[4], y[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) at(k + u * step, x[u], y[u]);
+    cfma<R>(r0, i0, x[0], y[0]);
+    cfma<R>(r1, i1, x[1], y[1]);
+    cfma<R>(r0, i0, x[2], y[2]);
+    cfma<R>(r1, i1, x[3], y[3]);
+  }
+  {
+    const Cx<R> zero = cmake<R>(R(0), R(0));
+    Cx<R> x[3] = {zero, zero, zero}, y[3] = {zero, zero, zero};
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+      if (k + u * step < a.K) at(k + u * step, x[u], y[u]);
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+      if (k + u * step < a.K) cfma<R>(u & 1 ? r1 : r0, u & 1 ? i1 : i0, x[u], y[u]);
+  }
+  sr = r0 + r1;
+  si = i0 + i1;
+}
+
+template <typename R>
+__device__ __forceinline__ void fine_store(const FineArgs<R>& a, long long idx, R sr, R si) {
+  Cx<R> v = cmake<R>(a.alpha * sr, a.alpha * si);
+  if (a.accumulate) {
+    const Cx<R> o = a.C[idx];
+    v.x += o.x;
+    v.y += o.y;
+  }
+  a.C[idx] = v;
+}
+
+template <typename R>
+__device__ __forceinline__ void fine_decode(const FineArgs<R>& a, unsigned o, unsigned& b, unsigned& m,
+                                            unsigned& n) {
+  const unsigned M = unsigned(a.M), N = unsigned(a.N);
+  if (a.n_fast) {
+    n = o % N;
+    o /= N;
+    m = o % M;
+    b = o / M;
+  } else {
+    m = o % M;
+    o /= M;
+    n = o % N;
+    b = o / N;
+  }
+}
+
+template <typename R>
+__global__ void __launch_bounds__(128) k_contract_fine(const FineArgs<R> a, unsigned total) {
+  const unsigned idx = blockIdx.x * 128u + threadIdx.x;
+  const unsigned o = idx >> a.ls_log, ks = idx & ((1u << a.ls_log) - 1u);
+  R sr = R(0), si = R(0);
+  unsigned b = 0, m = 0, n = 0;
+  const bool in = o < total;
+  if (in) {
+    fine_decode(a, o, b, m, n);
+    fine_sum<R>(a, a.A + a.aB[b] + a.aM[m], a.B + a.bB[b] + a.bN[n], int(ks), 1 << a.ls_log, sr, si);
+  }
+  for (int d = (1 << a.ls_log) >> 1; d > 0; d >>= 1) {
+    sr += __shfl_down_sync(0xffffffffu, sr, d);
+    si += __shfl_down_sync(0xffffffffu, si, d);
+  }
+  if (in && ks == 0) fine_store(a, a.cB[b] + a.cM[m] + a.cN[n], sr, si);
+}
+
+// One output per block: few outputs with long sums.
+template <typename R>
+__global__ void __launch_bounds__(256) k_contract_fine_block(const FineArgs<R> a) {
+  __shared__ R red[16];
+  unsigned b, m, n;
+  fine_decode(a, blockIdx.x, b, m, n);
+  R sr, si;
+  fine_sum<R>(a, a.A + a.aB[b] + a.aM[m], a.B + a.bB[b] + a.bN[n], int(threadIdx.x), 256, sr, si);
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) {
+    sr += __shfl_down_sync(0xffffffffu, sr, d);
+    si += __shfl_down_sync(0xffffffffu, si, d);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[2 * (threadIdx.x >> 5)] = sr;
+    red[2 * (threadIdx.x >> 5) + 1] = si;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  sr = red[0];
+  si = red[1];
+#pragma unroll
+  for (int w = 1; w < 8; ++w) {
+    sr += red[2 * w];
+    si += red[2 * w + 1];
+  }
+  fine_store(a, a.cB[b] + a.cM[m] + a.cN[n], sr, si);
+}
+
 }  // namespace
 
 template <typename R>
@@ -412,5 +527,30 @@ void launch_gemv(bool a_kc, const Cx<R>* A, long long aoff, const long long* aM,
 RTCC3_INST(float)
 RTCC3_INST(double)
 #undef RTCC3_INST
+
+void fine_split(long long outputs, long long K, int* ls_log, bool* block_wide) {
+  // fewer than about 8 warps' worth of outputs per SM and a long sum: a block
+  // each; else lanes until the GPU is covered (1024 lanes per SM) or a lane
+  // holds at most four terms
+  *block_wide = outputs * 32 < 152 * 256 && K >= 512;
+  int l = 0;
+  while (l < 5 && (outputs << l) < 152LL * 1024 && (K >> l) > 4) ++l;
+  *ls_log = l;
+}
+
+template <typename R>
+void launch_fine(const FineArgs<R>& a, cudaStream_t s) {
+  const long long total = (long long)a.M * a.N * a.nb;
+  if (a.block_wide) {
+    k_contract_fine_block<R><<<unsigned(total), 256, 0, s>>>(a);
+  } else {
+    const long long lanes = total << a.ls_log;
+    k_contract_fine<R><<<unsigned((lanes + 127) / 128), 128, 0, s>>>(a, unsigned(total));
+  }
+  RTCC3_CUDA(cudaGetLastError());
+}
+
+template void launch_fine<float>(const FineArgs<float>&, cudaStream_t);
+template void launch_fine<double>(const FineArgs<double>&, cudaStream_t);
 
 }  // namespace rtcc3

@@ -49,6 +49,29 @@ void launch_outer(const Cx<R>* A, long long aoff, const long long* aM, const lon
                   Cx<R>* C, long long coff, const long long* cM, const long long* cN, int M, int N,
                   double alpha, bool accumulate, cudaStream_t s);
 
+// Small products of any shape, spread over the whole GPU: 2^ls_log lanes of a
+// warp (or, block_wide, one block of 256 threads) share one output, each
+// summing every 2^ls_log-th k, joined by shuffles in a fixed order.  Offsets
+// along k are k * aks / k * bks when those are >= 0, else from the tables.
+// n_fast: consecutive outputs run along n (else along m).
+template <typename R>
+struct FineArgs {
+  const Cx<R>*A = nullptr, *B = nullptr;
+  Cx<R>* C = nullptr;
+  const long long *aM = nullptr, *aK = nullptr, *bN = nullptr, *bK = nullptr, *cM = nullptr,
+                  *cN = nullptr, *aB = nullptr, *bB = nullptr, *cB = nullptr;
+  int M = 1, N = 1, K = 1, nb = 1;
+  long long aks = -1, bks = -1;
+  int ls_log = 0;
+  bool n_fast = true, block_wide = false;
+  R alpha = R(1);
+  bool accumulate = false;
+};
+// Lane split of an outputs x K product (see FineArgs).
+void fine_split(long long outputs, long long K, int* ls_log, bool* block_wide);
+template <typename R>
+void launch_fine(const FineArgs<R>& a, cudaStream_t s);
+
 template <typename R>
 void launch_gemv(bool a_kc, const Cx<R>* A, long long aoff, const long long* aM, const long long* aK,
                  const Cx<R>* B, long long boff, const long long* bK, Cx<R>* C, long long coff,

@@ -17,6 +17,9 @@ constexpr int kBM = 64, kBN = 64, kBK = 16, kThreads = 256;
 constexpr int kSBM = 16, kSBK = 64;  // small-tile variant
 constexpr int kTBK = 8;               // thin (16 x 256) tiles
 constexpr int kTcMaxKbPerSplit = 16;  // K tiles per tensor-core accumulation chain
+// Complex multiply-adds up to which a product runs a few terms per lane over
+// the whole GPU (k_contract_fine) instead of in tiles.
+constexpr double kFineTermsF64 = 8e6, kFineTermsF32 = 2e6;
 constexpr size_t kLazyGradMin = 65536;  // gradients this large are not zero-filled up front
 
 // Division of 32-bit n < 2^31 by an invariant d >= 1 with one multiply-high
@@ -1173,7 +1176,7 @@ ContractPlan& Engine<R>::plan(const std::string& spec, const View& A, const View
   // 14440 24.5 -> 1.79 ms, 451 x 451 x 451 0.87 -> 0.09 ms; on the other side
   // of the line 10 x 10 x 5.5e6 (4.3 against 8.5 ms) and 144400 x 1 x 380
   // (0.42 against 0.67 ms) stay on the CUDA cores.
-  if (std::is_same<R, double>::value && NB == 1 && K >= 8) {
+  if (std::is_same<R, double>::value && NB == 1 && K >= 4) {
     const OzPlan oz = oz_plan(M, N, K);
     const double simt = 4.0 * double(M) * double(N) * double(K) / (2.0 * 152.0 * 0.85) + 4000.0;
     if (simt > oz.cost) {
@@ -1183,6 +1186,26 @@ ContractPlan& Engine<R>::plan(const std::string& spec, const View& A, const View
       plans_[key] = std::move(P);
       return ref;
     }
+  }
+  if (gk.size() <= 1) {
+    P->a_ks = gk.empty() ? 0 : gk[0].sa;
+    P->b_ks = gk.empty() ? 0 : gk[0].sb;
+  }
+  // small products: a few terms per lane over the whole GPU.  FP64: up to
+  // where the sliced form takes over; a 30 x 30 x 30 product takes 4 us against
+  // 45 us in tiles, 23 x 343 x 23 4 against 140 us.  FP32: up to about where
+  // the tiles' reuse of loads pays (19 x 475 x 19 3 against 7 us, at 4e6 terms
+  // both about 8 us).  A handful of outputs with a very long sum keeps the
+  // kernel that splits the sum over all SMs.
+  const bool long_few = M * N * NB * 32 < 152 * 256 && K > 8192;
+  const double terms = double(M) * double(N) * double(K) * double(NB);
+  const bool outer = NB == 1 && K == 1 && M * N >= 65536;
+  if (!outer && !long_few && terms <= (std::is_same<R, double>::value ? kFineTermsF64 : kFineTermsF32)) {
+    P->use_fine = true;
+    fine_split(M * N * NB, K, &P->fine_ls, &P->fine_block);
+    ContractPlan& ref = *P;
+    plans_[key] = std::move(P);
+    return ref;
   }
   // small outputs (held whole by every CTA, K split over the GPU) and single
   // long output columns get their own kernels
@@ -1346,6 +1369,30 @@ void Engine<R>::run_contract(const std::string& spec, double alpha, const View& 
   }
   if (P.use_oz) {
     run_contract_oz(P, alpha, pa, pb, pc, accumulate);
+    return;
+  }
+  if (P.use_fine) {
+    FineArgs<R> f;
+    f.A = pa;
+    f.B = pb;
+    f.C = pc;
+    f.aM = P.aM; f.aK = P.aK; f.bN = P.bN; f.bK = P.bK; f.cM = P.cM; f.cN = P.cN;
+    f.aB = P.aB; f.bB = P.bB; f.cB = P.cB;
+    f.M = P.M; f.N = P.N; f.K = P.K; f.nb = P.nb;
+    f.aks = P.a_ks;
+    f.bks = P.b_ks;
+    f.ls_log = P.fine_ls;
+    f.block_wide = P.fine_block;
+    f.n_fast = !P.c_unit_m;
+    f.alpha = R(alpha);
+    f.accumulate = accumulate;
+    const int pk = pbegin();
+    launch_fine<R>(f, stream_);
+    ++launches_;
+    const double mn = double(P.M) * P.N * P.nb;
+    pend(pk, sizeof(R) == 8 ? "contract_fine_c128" : "contract_fine_c64", 8.0 * mn * P.K,
+         (double(P.M) * P.K * P.nb + double(P.N) * P.K * P.nb + mn * (accumulate ? 2.0 : 1.0)) * sizeof(C),
+         cur_detail_);
     return;
   }
   if (P.kind != 0) {

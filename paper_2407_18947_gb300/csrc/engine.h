@@ -69,6 +69,10 @@ struct ContractPlan {
   bool use_tc = false, tc_swap = false;
   int tc_nsplit = 1, tc_kp = 0;
   bool tc_out = false;  // short sum bound by its output (two CTAs per SM)
+  // small products spread over the GPU, a few terms per lane (FineArgs)
+  bool use_fine = false, fine_block = false;
+  int fine_ls = 0;
+  long long a_ks = -1, b_ks = -1;  // strides along k when the sum is one index
   // FP64 products large enough for the sliced tensor-core form
   bool use_oz = false;
   bool c_unit_m = false;  // C's contiguous index is on the M side
