@@ -431,6 +431,8 @@ void launch_outer(const Cx<R>* A, long long aoff, const long long* aM, const lon
 }
 
 int small_output_config(long long M, long long N) {
+  if (M <= 6 && N <= 6) return kSmall6;
+  if (M <= 8 && N <= 8) return kSmall8;
   if (M <= 10 && N <= 10) return kSmall10;
   if (M <= 16 && N <= 16) return kSmall16;
   if (M <= 40 && N <= 40) return kSmall40;
@@ -441,9 +443,26 @@ int small_output_config(long long M, long long N) {
   return kSmallNone;
 }
 
+double small_output_tile(int cfg) {
+  switch (cfg) {
+    case kSmall6: return 36.0;
+    case kSmall8: return 64.0;
+    case kSmall10: return 100.0;
+    case kSmall16: return 256.0;
+    case kSmall40: return 1600.0;
+    case kSmall48: return 2304.0;
+    case kSmall64: return 4096.0;
+    case kSmallCol256: return 256.0;
+    case kSmallCol512: return 512.0;
+    default: return 0.0;
+  }
+}
+
 int small_output_bk(int cfg, int elem_bytes) {
   const bool d = elem_bytes == 16;
   switch (cfg) {
+    case kSmall6: return d ? SmallShape<double, 2, 1, 3, 6>::BK : SmallShape<float, 2, 1, 3, 6>::BK;
+    case kSmall8: return d ? SmallShape<double, 2, 2, 4, 4>::BK : SmallShape<float, 2, 2, 4, 4>::BK;
     case kSmall10: return d ? SmallShape<double, 2, 2, 5, 5>::BK : SmallShape<float, 2, 2, 5, 5>::BK;
     case kSmall16: return d ? SmallShape<double, 4, 4, 4, 4>::BK : SmallShape<float, 4, 4, 4, 4>::BK;
     case kSmall40: return d ? SmallShape<double, 8, 8, 5, 5>::BK : SmallShape<float, 8, 8, 5, 5>::BK;
@@ -462,6 +481,14 @@ void launch_reduce_small(int cfg, bool a_kc, bool b_kc, const Cx<R>* A, long lon
                          const long long* cM, const long long* cN, int M, int N, int K, int nsplit,
                          int kchunk, double alpha, bool accumulate, Cx<R>* part, cudaStream_t s) {
   switch (cfg) {
+    case kSmall6:
+      launch_cfg<R, 2, 1, 3, 6>(a_kc, b_kc, A, aoff, aM, aK, B, boff, bN, bK, C, coff, cM, cN, M, N, K,
+                                nsplit, kchunk, alpha, accumulate, part, s);
+      break;
+    case kSmall8:
+      launch_cfg<R, 2, 2, 4, 4>(a_kc, b_kc, A, aoff, aM, aK, B, boff, bN, bK, C, coff, cM, cN, M, N, K,
+                                nsplit, kchunk, alpha, accumulate, part, s);
+      break;
     case kSmall10:
       launch_cfg<R, 2, 2, 5, 5>(a_kc, b_kc, A, aoff, aM, aK, B, boff, bN, bK, C, coff, cM, cN, M, N, K,
                                 nsplit, kchunk, alpha, accumulate, part, s);

@@ -20,12 +20,14 @@ namespace rtcc3 {
 // Output-tile configurations of reduce_small (0 = not applicable).
 enum SmallCfg : int {
   kSmallNone = 0, kSmall48 = 1, kSmall16 = 2, kSmallCol256 = 3, kSmallCol512 = 4, kSmall64 = 5,
-  kSmall10 = 6, kSmall40 = 7
+  kSmall10 = 6, kSmall40 = 7, kSmall6 = 8, kSmall8 = 9
 };
 
 // Configuration for an M x N output (N <= M expected; returns kSmallNone
 // when the shape is not small).
 int small_output_config(long long M, long long N);
+// Outputs of a configuration's tile (what it computes, padding included).
+double small_output_tile(int cfg);
 // Depth of one K slice for a configuration (chunks are multiples of it).
 int small_output_bk(int cfg, int elem_bytes);
 

@@ -1171,14 +1171,18 @@ ContractPlan& Engine<R>::plan(const std::string& spec, const View& A, const View
   // FP64 products above a few million multiply-adds: sliced products on the
   // tensor cores (oz_gemm.h).  Both sides in SM clocks: the CUDA cores do two
   // FP64 multiply-adds per SM and clock (four per complex one, 85 % of that
-  // rate at best), the sliced form costs what its plan estimates.  Measured,
-  // CUDA cores against sliced: 3800 x 14440 x 48 17.6 -> 2.17 ms, 3800 x 38 x
-  // 14440 24.5 -> 1.79 ms, 451 x 451 x 451 0.87 -> 0.09 ms; on the other side
-  // of the line 10 x 10 x 5.5e6 (4.3 against 8.5 ms) and 144400 x 1 x 380
-  // (0.42 against 0.67 ms) stay on the CUDA cores.
+  // rate at best, and small outputs are padded to their tile), the sliced form
+  // costs what its plan estimates.  Measured, CUDA cores against sliced:
+  // 3800 x 14440 x 48 17.6 -> 1.35 ms, 3800 x 38 x 14440 24.5 -> 1.05 ms, 38 x
+  // 38 x 1.4e6 15.6 -> 3.0 ms, 451 x 451 x 451 0.87 -> 0.054 ms; on the other
+  // side of the line 10 x 10 x 5.5e6 (4.33 against 4.36 ms) and 144400 x 1 x
+  // 380 (0.42 against 0.46 ms) stay on the CUDA cores.
   if (std::is_same<R, double>::value && NB == 1 && K >= 4) {
     const OzPlan oz = oz_plan(M, N, K);
-    const double simt = 4.0 * double(M) * double(N) * double(K) / (2.0 * 152.0 * 0.85) + 4000.0;
+    double terms = double(M) * double(N) * double(K);
+    if (K >= 256 && std::max(M, N) <= 64 && terms > kFineTermsF64)
+      terms = double(K) * small_output_tile(small_output_config(std::max(M, N), std::min(M, N)));
+    const double simt = 4.0 * terms / (2.0 * 152.0 * 0.85) + 4000.0;
     if (simt > oz.cost) {
       P->use_oz = true;
       P->oz = oz;

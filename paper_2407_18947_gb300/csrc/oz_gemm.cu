@@ -12,9 +12,11 @@
 //
 // No FP64 instruction is used on the way to a first result: conversion and
 // joining are integer work, because an SM has 64 times fewer FP64 lanes than
-// integer ones.  Bound by the integer work and its latencies (3800 x 14440 x
-// 48: ALU pipe 42 % busy, tensor pipe 15 %, 50000 clocks per tile; 17.6 ms on
-// the FP64 cores before, 2.17 ms now).
+// integer ones.  The code is kept small (rolled loops): fetched once per tile,
+// 85 KB of straight-line code took longer than the work.  Bound by the
+// integer work and load latencies (3800 x 14440 x 48: 52000 warp instructions
+// and 31000 clocks per tile, of which the MMAs take 7000; 17.6 ms on the FP64
+// cores, 1.35 ms here).
 #include "oz_gemm.h"
 
 #include <cuda_fp16.h>
@@ -33,7 +35,7 @@ constexpr int kSl = 8;              // digits
 constexpr int kRows = 128;          // A rows per tile
 constexpr int kKC = 16;             // complex k per stage (64-byte FP16 rows)
 constexpr int kWorkers = 16;        // worker warps
-constexpr int kSegMax = 128;        // complex k per segment (256 real: see oz_gemm.h)
+constexpr int kSegMax = 128;        // complex k per segment (256 real: see oz_gemm.h; a power of two)
 constexpr unsigned long long kBias = 0x8080808080808080ULL;
 
 template <int NT>
@@ -42,9 +44,10 @@ struct OzSmem {
   static constexpr int kStage = kSl * (kASlice + kBSlice);
   static constexpr int kPitch = NT / 2 + 1;  // complex per staged output row
   static constexpr int kBarOff = 2 * kStage;
-  static constexpr int kExpOff = kBarOff + 64;                 // row exponents
-  static constexpr int kTotal = kExpOff + (kRows + NT / 2) * 4 + 1024;
-  static constexpr int kCols = kSl * NT < 32 ? 32 : kSl * NT;  // TMEM columns
+  static constexpr int kExpOff = kBarOff + 64;  // row exponents, two segments
+  static constexpr int kTabOff = kExpOff + 2 * (kRows + 32) * 4;  // k offsets (two segments), output offsets
+  static constexpr int kTotal = kTabOff + (4 * kSegMax + kRows + NT / 2) * 8 + 1024;
+  static constexpr int kCols = NT <= 16 ? 128 : (NT <= 32 ? 256 : 512);  // TMEM columns (a power of two)
   static_assert(kRows * kPitch * 16 <= 2 * kStage, "output staging");
   static_assert(kTotal <= 232448, "shared memory per CTA");
 };
@@ -69,97 +72,182 @@ __device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t a, uint64_t b, u
       : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld4(uint32_t t, uint32_t (&r)[4]) {
+__device__ __forceinline__ void tmem_ld(uint32_t t, uint32_t (&r)[4]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(t));
 }
 
+__device__ __forceinline__ void tmem_ld(uint32_t t, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+                 "=r"(r[7])
+               : "r"(t));
+}
+
 // |x| as a sortable word whose top 11 bits are its exponent field.
-__device__ __forceinline__ uint32_t hiabs(double x) { return uint32_t(__double2hiint(x)) & 0x7fffffffu; }
+__device__ __forceinline__ uint32_t hiabs(uint32_t hi) { return hi & 0x7fffffffu; }
 
-// a (|a| < 2^(F - 1022)) as the biased digits of its 62-bit fixed-point form:
-// byte 7 - s of the result is digit s plus 128.
-__device__ __forceinline__ unsigned long long digits(double a, int F) {
+// |a| (below 2^(F - 1022), F >= 64) as the biased digits of its 62-bit
+// fixed-point form: byte 7 - s is digit s of |a| plus 128.  Elements below
+// 2^-62 of the bound (zeros and subnormals among them) have zero digits.
+__device__ __forceinline__ void digits(double a, int F, uint32_t& yh, uint32_t& yl) {
   const uint32_t hi = uint32_t(__double2hiint(a)), lo = uint32_t(__double2loint(a));
-  const int ex = int((hi >> 20) & 0x7ffu);
+  const int n = min(F - int(hiabs(hi) >> 20), 63);
   const unsigned long long m =
-      (static_cast<unsigned long long>((hi & 0xfffffu) | (ex ? 0x100000u : 0u)) << 32) | lo;
-  const int n = min(max(F - max(ex, 1), 0), 63);
-  const unsigned long long x = (((m << 10) >> n) + 1ULL) >> 1;
-  return (hi >> 31) ? kBias - x : kBias + x;
+      (static_cast<unsigned long long>((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+  const unsigned long long y = ((m << 9) >> n) + kBias;
+  yh = uint32_t(y >> 32);
+  yl = uint32_t(y);
 }
 
-// Digit s of (re, im) as a pair of halves (1024 + u has the bits 0x6400 | u).
-template <int S>
-__device__ __forceinline__ uint32_t digit_pair(unsigned long long yr, unsigned long long yi) {
-  const uint32_t r = S < 4 ? uint32_t(yr >> 32) : uint32_t(yr);
-  const uint32_t i = S < 4 ? uint32_t(yi >> 32) : uint32_t(yi);
-  constexpr uint32_t b = 3 - (S & 3);
-  uint32_t u = __byte_perm(r, i, b | (b << 4) | ((4 + b) << 8) | ((4 + b) << 12));
-  u = (u & 0x00ff00ffu) | 0x64006400u;
-  const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&u),
-                            __half2(__ushort_as_half(0x6480), __ushort_as_half(0x6480)));
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
+// The eight digits of a complex number as pairs of halves (re, im), signs
+// applied: u has the bits 0x6400 | byte = 1024 + byte, so one FMA by (+-1, +-1)
+// with the addend -+1152 gives the digit.
+struct DigitPairs {
+  uint32_t q[4];  // interleaved bytes (re_s, im_s, re_s+1, im_s+1), s = 0, 2, 4, 6
+  __half2 sg, c;
+  __device__ __forceinline__ DigitPairs(double2 z, int F) {
+    uint32_t rh, rl, ih, il;
+    digits(z.x, F, rh, rl);
+    digits(z.y, F, ih, il);
+    q[0] = __byte_perm(rh, ih, 0x6273);  // bytes 3, 7, 2, 6 from low to high
+    q[1] = __byte_perm(rh, ih, 0x4051);
+    q[2] = __byte_perm(rl, il, 0x6273);
+    q[3] = __byte_perm(rl, il, 0x4051);
+    const uint32_t sr = uint32_t(__double2hiint(z.x)), si = uint32_t(__double2hiint(z.y));
+    const uint32_t w = (__byte_perm(sr, si, 0x7030) & 0x80008000u) | 0x3c003c00u;
+    sg = *reinterpret_cast<const __half2*>(&w);
+    c = __hmul2(sg, __half2(__ushort_as_half(0xe480), __ushort_as_half(0xe480)));  // -1152
+  }
+  template <int S>
+  __device__ __forceinline__ uint32_t get() const {
+    const uint32_t u = __byte_perm(q[S >> 1], 0x64u, (S & 1) ? 0x4342 : 0x4140);
+    const __half2 h = __hfma2(*reinterpret_cast<const __half2*>(&u), sg, c);
+    return *reinterpret_cast<const uint32_t*>(&h);
+  }
+};
 
 __device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
   asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
 template <int S, int STRIDE>
-__device__ __forceinline__ void store_a(uint32_t addr, unsigned long long yr, unsigned long long yi) {
+__device__ __forceinline__ void store_a(uint32_t addr, const DigitPairs& d) {
   if constexpr (S < kSl) {
-    sts32(addr + S * STRIDE, digit_pair<S>(yr, yi));
-    store_a<S + 1, STRIDE>(addr, yr, yi);
+    sts32(addr + S * STRIDE, d.template get<S>());
+    store_a<S + 1, STRIDE>(addr, d);
   }
 }
 
-// Both rows of B's embedding, (re, -im) at row 2n and (im, re) at row 2n + 1;
-// h: which of the two is stored first (lanes of both kinds share a store
-// instruction without a bank conflict).
+// One row of B's embedding: (re, -im) at row 2n (odd = false), (im, re) at row
+// 2n + 1.
+struct RowPairs {
+  uint32_t sel0, sel1;  // byte selectors of the even and odd digits
+  __half2 sg, c;
+  __device__ __forceinline__ RowPairs(const DigitPairs& d, bool odd) {
+    sel0 = odd ? 0x4041 : 0x4140;
+    sel1 = odd ? 0x4243 : 0x4342;
+    const uint32_t w = *reinterpret_cast<const uint32_t*>(&d.sg);
+    const uint32_t x = odd ? __byte_perm(w, w, 0x1032) : w ^ 0x80000000u;
+    sg = *reinterpret_cast<const __half2*>(&x);
+    c = __hmul2(sg, __half2(__ushort_as_half(0xe480), __ushort_as_half(0xe480)));
+  }
+};
+
 template <int S, int STRIDE>
-__device__ __forceinline__ void store_b(uint32_t addr, uint32_t h, unsigned long long yr,
-                                        unsigned long long yi) {
+__device__ __forceinline__ void store_b(uint32_t addr, const DigitPairs& d, const RowPairs& r) {
   if constexpr (S < kSl) {
-    const uint32_t d = digit_pair<S>(yr, yi);
-    const uint32_t even = d ^ 0x80000000u, odd = __byte_perm(d, d, 0x1032);
-    sts32(addr + S * STRIDE + (h ? 64 : 0), h ? odd : even);
-    sts32(addr + S * STRIDE + (h ? 0 : 64), h ? even : odd);
-    store_b<S + 1, STRIDE>(addr, h, yr, yi);
+    const uint32_t u = __byte_perm(d.q[S >> 1], 0x64u, (S & 1) ? r.sel1 : r.sel0);
+    const __half2 h = __hfma2(*reinterpret_cast<const __half2*>(&u), r.sg, r.c);
+    sts32(addr + S * STRIDE, *reinterpret_cast<const uint32_t*>(&h));
+    store_b<S + 1, STRIDE>(addr, d, r);
   }
 }
 
-// sum_g v_g 2^(56 - 8 g) 2^E, the v_g integers held in FP32, rounded to nearest.
-// ash, neg: times 2^ash and -1.
-__device__ __forceinline__ double join(const uint32_t* v, int E, int neg) {
-  auto iv = [&](int g) { return (long long)__float2int_rn(__uint_as_float(v[g])); };
-  long long hi = iv(0) * (1LL << 24) + iv(1) * (1LL << 16) + iv(2) * 256 + iv(3);
-  const long long lo = iv(4) * (1LL << 24) + iv(5) * (1LL << 16) + iv(6) * 256 + iv(7);
-  // value = hi 2^32 + lo as a 96-bit integer
-  hi += lo >> 32;
-  uint32_t w0 = uint32_t(lo);
-  if (hi < 0) {
-    neg ^= 1;
-    w0 = 0u - w0;
-    hi = w0 ? ~hi : -hi;
-  }
-  uint32_t w1 = uint32_t(hi), w2 = uint32_t(static_cast<unsigned long long>(hi) >> 32);
-  int e = E + 32;
+constexpr int kZeroExp = 1 << 16;  // row exponent that makes every digit zero
+constexpr int kNanExp = 1 << 18;  // exponent of a row with a non-finite element
+
+__device__ __forceinline__ double join_rare(uint32_t w2, uint32_t w1, uint32_t w0, int e, uint32_t sign) {
+  if (e >= kNanExp / 2) return __longlong_as_double(0x7ff8000000000000LL);
   if (w2 == 0) { w2 = w1; w1 = w0; w0 = 0; e -= 32; }
   if (w2 == 0) { w2 = w1; w1 = w0; w0 = 0; e -= 32; }
   if (w2 == 0) return 0.0;
   const int lz = __clz(w2);
   const unsigned long long top =
       (static_cast<unsigned long long>(__funnelshift_l(w1, w2, lz)) << 32) | __funnelshift_l(w0, w1, lz);
-  const unsigned long long t = (top >> 11) + ((top >> 10) & 1ULL);  // 53 bits
+  const unsigned long long t = (top >> 11) + ((top >> 10) & 1ULL);
   const int field = e - lz + 63 + 1023;
-  unsigned long long bits;
-  if (field <= 0) bits = 0ULL;
-  else bits = (static_cast<unsigned long long>(field - 1) << 52) + t;
+  unsigned long long bits = 0ULL;  // below the normal range: zero
+  if (field > 0) bits = (static_cast<unsigned long long>(field - 1) << 52) + t;
   if (field >= 2047 || bits > 0x7ff0000000000000ULL) bits = 0x7ff0000000000000ULL;
-  bits |= static_cast<unsigned long long>(neg) << 63;
-  return __longlong_as_double((long long)bits);
+  return __longlong_as_double((long long)(bits | (static_cast<unsigned long long>(sign & 0x80000000u) << 32)));
+}
+
+// (hi 2^32 + lo) 2^16 as sign (all ones or 0) and 96-bit magnitude w2:w1:w0
+// (|hi| < 2^47).
+__device__ __forceinline__ uint32_t magnitude(long long hi, long long lo, uint32_t& w2, uint32_t& w1,
+                                              uint32_t& w0) {
+  hi += int(lo >> 32);
+  const uint32_t s = uint32_t(hi >> 63);
+  const uint32_t h1 = uint32_t(static_cast<unsigned long long>(hi) >> 32), h0 = uint32_t(hi), l = uint32_t(lo);
+  w2 = __byte_perm(h0, h1, 0x5432) ^ s;
+  w1 = __byte_perm(l, h0, 0x5432) ^ s;
+  w0 = (l << 16) ^ s;
+  asm("sub.cc.u32 %0, %0, %3;\n\tsubc.cc.u32 %1, %1, %3;\n\tsubc.u32 %2, %2, %3;"
+      : "+r"(w0), "+r"(w1), "+r"(w2)
+      : "r"(s));
+  return s;
+}
+
+// join() of any accumulators: above 2^22, zero sums, results outside the
+// normal range, rows with a non-finite element.
+__device__ __noinline__ double join_any(float v0, float v1, float v2, float v3, float v4, float v5,
+                                        float v6, float v7, int E, uint32_t sgn) {
+  auto iv = [](float v) { return (long long)__float2int_rn(v); };
+  uint32_t w2, w1, w0;
+  const uint32_t s = magnitude((iv(v0) << 24) + (iv(v1) << 16) + (iv(v2) << 8) + iv(v3),
+                               (iv(v4) << 24) + (iv(v5) << 16) + (iv(v6) << 8) + iv(v7), w2, w1, w0);
+  return join_rare(w2, w1, w0, E + 16, s ^ sgn);
+}
+
+// sum_g v_g 2^(56 - 8 g) 2^E, the v_g integers held in FP32, rounded to
+// nearest; sgn: all ones for the negative.  Integers up to 2^22 (nearly all; v0
+// and v1 always) leave FP32 by an addition that puts them into the mantissa:
+// the conversion instruction has an eighth of that rate.
+__device__ __forceinline__ double join(const float (&v)[kSl], int E, uint32_t sgn) {
+  const float big = fmaxf(fmaxf(fmaxf(fabsf(v[2]), fabsf(v[3])), fabsf(v[4])),
+                          fmaxf(fmaxf(fabsf(v[5]), fabsf(v[6])), fabsf(v[7])));
+  // pairs v_g 256 + v_(g+1): below 2^31
+  auto two = [&](int g) {
+    const uint32_t p = __float_as_uint(v[g] + 12582912.0f), q = __float_as_uint(v[g + 1] + 12582912.0f);
+    return int(p * 256u + q - 0x4b400000u * 257u);
+  };
+  uint32_t w2, w1, w0;
+  const uint32_t sign = magnitude((long long)two(0) * 65536 + two(2), (long long)two(4) * 65536 + two(6),
+                                  w2, w1, w0) ^ sgn;
+  const int lz = __clz(w2);
+  const uint32_t th = __funnelshift_l(w1, w2, lz), tl = __funnelshift_l(w0, w1, lz);
+  const int field = E - lz + 16 + 63 + 1023;
+  if (big > 4194304.0f || w2 == 0 || unsigned(field - 1) >= 2045u)
+    return join_any(v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7], E, sgn);
+  // 53 bits of th:tl (top bit set), rounded; the carry runs into the exponent
+  unsigned long long t = ((static_cast<unsigned long long>(th) << 32) | tl) >> 11;
+  t += (tl >> 10) & 1u;
+  t += static_cast<unsigned long long>(uint32_t(field - 1) << 20 | (sign & 0x80000000u)) << 32;
+  return __longlong_as_double((long long)t);
+}
+
+constexpr int kMinExp = 64;  // smallest row exponent (2^-958): digits() needs it
+
+// Larger of |re| and |im| of a row element, as its high word.
+__device__ __forceinline__ uint32_t row_word(const double2* p) {
+  const uint32_t* w = reinterpret_cast<const uint32_t*>(p);
+  return max(hiabs(__ldg(w + 1)), hiabs(__ldg(w + 3)));
+}
+
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
 struct OzArgs {
@@ -168,7 +256,8 @@ struct OzArgs {
   double2* C;      // already moved by its offset; the partials when nsplit > 1
   int M, N, K;
   int seg, nseg, spc;
-  int ash, neg;    // alpha = (neg ? -1 : 1) 2^ash alpha_rest
+  int ash;         // alpha = (neg ? -1 : 1) 2^ash alpha_rest, neg = all ones or 0
+  uint32_t neg;
   double alpha_rest;
   int accumulate, to_part, c_m;
   int* err;
@@ -180,14 +269,17 @@ __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs 
   using L = OzSmem<NT>;
   constexpr int NB = NT / 2;   // complex columns
   constexpr int CPT = NT / 4;  // real columns a worker thread reads back
+  constexpr int CU = CPT % 8 == 0 ? 8 : 4;  // at a time
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::kBarOff);
   uint64_t *full = bars, *empty = bars + 2, *done = bars + 4, *fin = bars + 5;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 6);
   int* sEA = reinterpret_cast<int*>(smem + L::kExpOff);
-  int* sEB = sEA + kRows;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  long long* sK = reinterpret_cast<long long*>(smem + L::kTabOff);  // k offsets: A, then B
+  long long* sCM = sK + 4 * kSegMax;
+  long long* sCN = sCM + kRows;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
   const int m0 = blockIdx.y * kRows, n0 = blockIdx.x * NB;
   const int s0 = blockIdx.z * P.spc, s1 = min(P.nseg, s0 + P.spc);
 
@@ -205,6 +297,9 @@ __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs 
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tmem_slot)), "r"(L::kCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  } else if (!P.to_part) {
+    if (tid < kRows) sCM[tid] = m0 + tid < P.M ? P.cM[m0 + tid] : 0;
+    else if (tid < kRows + NB) sCN[tid - kRows] = n0 + tid - kRows < P.N ? P.cN[n0 + tid - kRows] : 0;
   }
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -250,195 +345,220 @@ __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs 
     }
   } else {
     const int w = warp;
-    // rows this thread reads: AKC two rows x 16 k per warp access, else 8 rows x 4 k
-    constexpr int UA = 4;
-    long long arow[AKC ? UA : 1];
-    bool aok[AKC ? UA : 1];
-    if (AKC) {
+    // Element u of a thread in a stage.  A: warp w owns rows 8 w .. + 7; one
+    // access covers two rows x 16 k (AKC) or 8 rows x 4 k.  B: 32 rows.
+    constexpr int UA = 4, RA = AKC ? UA : 1;
+    auto ar = [&](int u) { return AKC ? 8 * w + 2 * u + (lane >> 4) : 8 * w + (lane & 7); };
+    auto ak = [&](int u) { return AKC ? (lane & 15) : 4 * u + (lane >> 3); };
+    auto br = [&](int) { return BKC ? 2 * w + (lane >> 4) : 8 * (w >> 2) + (lane & 7); };
+    auto bk = [&](int) { return BKC ? (lane & 15) : 4 * (w & 3) + (lane >> 3); };
+    // Rows and k outside the matrix repeat the last one inside: such rows of the
+    // result are not stored, and B's digits are zero beyond the last k.
+    const char* arow[RA];
 #pragma unroll
-      for (int u = 0; u < UA; ++u) {
-        const int m = m0 + 8 * w + 2 * u + (lane >> 4);
-        aok[u] = m < P.M;
-        arow[u] = aok[u] ? P.aM[m] : 0;
-      }
-    } else {
-      const int m = m0 + 8 * w + (lane & 7);
-      aok[0] = m < P.M;
-      arow[0] = aok[0] ? P.aM[m] : 0;
-    }
-    const int bn = BKC ? 2 * w + (lane >> 4) : 8 * (w >> 2) + (lane & 7);
-    const int bk = BKC ? (lane & 15) : 4 * (w & 3) + (lane >> 3);
-    const bool bact = bn < NB;
-    const bool bok = bact && n0 + bn < P.N;
-    const long long brow = bok ? P.bN[n0 + bn] : 0;
+    for (int u = 0; u < RA; ++u)
+      arow[u] = reinterpret_cast<const char*>(P.A + P.aM[min(m0 + ar(u), P.M - 1)]);
+    const char* brow = reinterpret_cast<const char*>(P.B + P.bN[min(n0 + br(0), P.N - 1)]);
+    auto aat = [&](int u, long long off) {
+      return reinterpret_cast<const double2*>(arow[AKC ? u : 0] + off);
+    };
+    auto bat = [&](long long off) { return reinterpret_cast<const double2*>(brow + off); };
+    // a warp whose rows all lie outside the matrix only clears them once
+    const bool wact = m0 + 8 * w < P.M;
     const double2 zero = make_double2(0.0, 0.0);
-    double acc[CPT];
+    auto table = [&](int sg) {  // k offsets of a segment, in bytes
+      if (tid >= 2 * kSegMax) return;
+      const int k = min(sg * P.seg + min(tid & (kSegMax - 1), P.seg - 1), P.K - 1);
+      sK[(sg & 1) * 2 * kSegMax + tid] = 16 * (tid < kSegMax ? P.aK[k] : P.bK[k]);
+    };
+    table(s0);
     int it = 0;
+#pragma unroll 1
     for (int sg = s0; sg < s1; ++sg) {
-      const int kb = sg * P.seg, ke = min(P.K, kb + P.seg);
-      // ---- exponents of the segment's rows ------------------------------------
-      if (threadIdx.x < NB) sEB[threadIdx.x] = 1;
+      const int kb = sg * P.seg, klen = min(P.K, kb + P.seg) - kb;
+      const long long* tk = sK + (sg & 1) * 2 * kSegMax;
+      int* eA = sEA + (sg & 1) * (kRows + 32);
+      int* eB = eA + kRows;
+      if (tid < NB) eB[tid] = kMinExp;
       asm volatile("bar.sync 1, %0;" ::"r"(32 * kWorkers) : "memory");
-      int fa[AKC ? UA : 1];
-      if (AKC) {
-        uint32_t mx[UA] = {0, 0, 0, 0};
-#pragma unroll 2
-        for (int k = kb + (lane & 15); k < ke; k += 16) {
-          const long long ok_ = P.aK[k];
+      auto fetch = [&](int c, double2 (&na)[UA], double2& nb) {
 #pragma unroll
-          for (int u = 0; u < UA; ++u) {
-            const double2 x = aok[u] ? P.A[arow[u] + ok_] : zero;
-            mx[u] = max(mx[u], max(hiabs(x.x), hiabs(x.y)));
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < UA; ++u) {
-#pragma unroll
-          for (int d = 8; d > 0; d >>= 1) mx[u] = max(mx[u], __shfl_xor_sync(0xffffffffu, mx[u], d));
-          fa[u] = max(int(mx[u] >> 20), 1);
-          if ((lane & 15) == 0) sEA[8 * w + 2 * u + (lane >> 4)] = fa[u];
-        }
-      } else {
-        uint32_t mx = 0;
-#pragma unroll 8
-        for (int k = kb + (lane >> 3); k < ke; k += 4) {
-          const double2 x = aok[0] ? P.A[arow[0] + P.aK[k]] : zero;
-          mx = max(mx, max(hiabs(x.x), hiabs(x.y)));
-        }
-        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
-        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
-        fa[0] = max(int(mx >> 20), 1);
-        if (lane < 8) sEA[8 * w + lane] = fa[0];
-      }
-      if (bok) {
-        uint32_t mx = 0;
-#pragma unroll 4
-        for (int k = kb + bk; k < ke; k += 16) {
-          const double2 x = P.B[brow + P.bK[k]];
-          mx = max(mx, max(hiabs(x.x), hiabs(x.y)));
-        }
-        atomicMax(&sEB[bn], int(mx >> 20));
-      }
-      asm volatile("bar.sync 1, %0;" ::"r"(32 * kWorkers) : "memory");
-      const int fb = bact ? sEB[bn] : 1;
-
-      // ---- conversion, one stage ahead of the MMAs ------------------------------
-      const int nch = (ke - kb + kKC - 1) / kKC;
-      double2 na[UA], nbv;
-      auto fetch = [&](int c) {
-        const int k0 = kb + c * kKC;
-        if (AKC) {
-          const int k = k0 + (lane & 15);
-          const long long o = k < ke ? P.aK[k] : 0;
-#pragma unroll
-          for (int u = 0; u < UA; ++u) na[u] = (aok[u] && k < ke) ? P.A[arow[u] + o] : zero;
-        } else {
-#pragma unroll
-          for (int u = 0; u < UA; ++u) {
-            const int k = k0 + 4 * u + (lane >> 3);
-            na[u] = (aok[0] && k < ke) ? P.A[arow[0] + P.aK[k]] : zero;
-          }
-        }
-        const int k = k0 + bk;
-        nbv = (bok && k < ke) ? P.B[brow + P.bK[k]] : zero;
+        for (int u = 0; u < UA; ++u) na[u] = *aat(u, tk[c * kKC + ak(u)]);
+        nb = *bat(tk[kSegMax + c * kKC + bk(0)]);
       };
-      fetch(0);
-      for (int c = 0; c < nch; ++c, ++it) {
+      // the first two stages' elements, used for the exponents too
+      double2 na0[UA], na1[UA], nb0, nb1;
+      fetch(0, na0, nb0);
+      fetch(1, na1, nb1);
+      // ---- exponents of the segment's rows (later stages: read for them only,
+      // the conversion finds them in L2 again) ------------------------------------
+      int fa[RA], fb;
+      {
+        uint32_t ma[RA], mb = 0;
+#pragma unroll
+        for (int u = 0; u < RA; ++u) ma[u] = 0;
+#pragma unroll 1
+        for (int k0 = 2 * kKC; k0 < klen; k0 += 3 * kKC) {
+          uint32_t x[3][UA], y[3];
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+#pragma unroll
+            for (int u = 0; u < UA; ++u) x[c][u] = row_word(aat(u, tk[k0 + c * kKC + ak(u)]));
+            y[c] = row_word(bat(tk[kSegMax + k0 + c * kKC + bk(0)]));
+          }
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+#pragma unroll
+            for (int u = 0; u < UA; ++u) ma[AKC ? u : 0] = max(ma[AKC ? u : 0], x[c][u]);
+            mb = max(mb, y[c]);
+          }
+        }
+        auto word = [](double2 z) {
+          return max(hiabs(uint32_t(__double2hiint(z.x))), hiabs(uint32_t(__double2hiint(z.y))));
+        };
+#pragma unroll
+        for (int u = 0; u < UA; ++u)
+          ma[AKC ? u : 0] = max(ma[AKC ? u : 0], max(word(na0[u]), word(na1[u])));
+        mb = max(mb, max(word(nb0), word(nb1)));
+#pragma unroll
+        for (int u = 0; u < RA; ++u) {
+          // the lanes of one row: 16 neighbours (AKC) or every eighth lane
+#pragma unroll
+          for (int d = AKC ? 8 : 16; d >= (AKC ? 1 : 8); d >>= 1)
+            ma[u] = max(ma[u], __shfl_xor_sync(0xffffffffu, ma[u], d));
+          fa[u] = max(int(ma[u] >> 20), kMinExp);
+          if (AKC ? (lane & 15) == 0 : lane < 8) eA[ar(u)] = fa[u] == 2047 ? kNanExp : fa[u];
+        }
+#pragma unroll
+        for (int d = BKC ? 8 : 16; d >= (BKC ? 1 : 8); d >>= 1)
+          mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, d));
+        const int f = int(mb >> 20);
+        if ((BKC ? (lane & 15) == 0 : lane < 8) && br(0) < NB)
+          atomicMax(&eB[br(0)], f == 2047 ? kNanExp : f);
+      }
+      asm volatile("bar.sync 1, %0;" ::"r"(32 * kWorkers) : "memory");
+      fb = br(0) < NB ? min(eB[br(0)], 2047) : kMinExp;
+      if (sg + 1 < s1) table(sg + 1);
+
+      // ---- conversion: elements fetched two stages ahead ----------------------------
+      const int nch = (klen + kKC - 1) / kKC;
+      auto convert = [&](int c, double2 (&na)[UA], double2& nb) {
         const int st = it & 1;
-        double2 ca[UA];
+        if (sg + 1 < s1 && wact && c > 0) {
+          // the same places of the next segment, for its exponents
 #pragma unroll
-        for (int u = 0; u < UA; ++u) ca[u] = na[u];
-        const double2 cb = nbv;
-        if (c + 1 < nch) fetch(c + 1);
+          for (int u = 0; u < UA; ++u) {
+            const int k = kb + P.seg + (c - 1) * kKC + ak(u);
+            if (k < P.K) prefetch_l2(aat(u, 16 * P.aK[k]));
+          }
+        }
         if (it >= 2 && ok) ok = mbar_wait(smem_u32(&empty[st]), ((it >> 1) - 1) & 1, P.budget);
-        if (!ok) continue;
-        const uint32_t sa = smem_u32(smem + st * L::kStage), sb = sa + kSl * L::kASlice;
+        if (ok) {
+          const uint32_t sa = smem_u32(smem + st * L::kStage), sb = sa + kSl * L::kASlice;
+          if (wact || it < 2) {
 #pragma unroll
-        for (int u = 0; u < UA; ++u) {
-          const int r = AKC ? 8 * w + 2 * u + (lane >> 4) : 8 * w + (lane & 7);
-          const int k = AKC ? (lane & 15) : 4 * u + (lane >> 3);
-          const uint32_t at = sa + uint32_t(r * 64 + (((k >> 2) ^ ((r >> 1) & 3)) << 4) + (k & 3) * 4);
-          const int F = AKC ? fa[u] : fa[0];
-          store_a<0, L::kASlice>(at, digits(ca[u].x, F), digits(ca[u].y, F));
+            for (int u = 0; u < UA; ++u) {
+              const int r = ar(u), k = ak(u);
+              const uint32_t at = sa + uint32_t(r * 64 + (((k >> 2) ^ ((r >> 1) & 3)) << 4) + (k & 3) * 4);
+              store_a<0, L::kASlice>(at, DigitPairs(na[u], fa[AKC ? u : 0]));
+            }
+          }
+          const int n = br(0), k = bk(0);
+          if (n < NB) {
+            const uint32_t at = sb + uint32_t(n * 128 + (((k >> 2) ^ (n & 3)) << 4) + (k & 3) * 4);
+            const DigitPairs d(nb, c * kKC + k < klen ? fb : kZeroExp);
+            // lanes of both kinds share a store instruction without a bank conflict
+            const bool h = BKC ? (lane >> 4) != 0 : ((n >> 2) & 1) != 0;
+            store_b<0, L::kBSlice>(at + (h ? 64 : 0), d, RowPairs(d, h));
+            store_b<0, L::kBSlice>(at + (h ? 0 : 64), d, RowPairs(d, !h));
+          }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&full[st]));
         }
-        if (bact) {
-          const uint32_t at = sb + uint32_t(bn * 128 + (((bk >> 2) ^ (bn & 3)) << 4) + (bk & 3) * 4);
-          store_b<0, L::kBSlice>(at, uint32_t(BKC ? (lane >> 4) : ((bn >> 2) & 1)), digits(cb.x, fb),
-                                 digits(cb.y, fb));
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&full[st]));
+        ++it;
+        if (c + 2 < nch) fetch(c + 2, na, nb);
+      };
+#pragma unroll 1
+      for (int c = 0; c < nch; c += 2) {
+        convert(c, na0, nb0);
+        if (c + 1 < nch) convert(c + 1, na1, nb1);
       }
 
       // ---- read the accumulators back ---------------------------------------------
       if (ok) ok = mbar_wait(smem_u32(done), (sg - s0) & 1, P.budget);
       ok = __all_sync(0xffffffffu, ok);
-      if (ok) {
+      const int q = w & 3, c0 = (w >> 2) * CPT;
+      // a staged tile overwrites the stages: every MMA has completed, and no
+      // warp converts any more (a staged tile is its CTA's only segment)
+      double* stg = reinterpret_cast<double*>(smem) + (q * 32 + lane) * (2 * L::kPitch) + c0;
+      const int m = m0 + q * 32 + lane;
+      double2* prow = P.C + ((long long)sg * P.M + m) * P.N + n0 + (c0 >> 1);
+      if (ok && m0 + q * 32 < P.M && 2 * n0 + c0 < 2 * P.N) {  // else: no output here
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const int q = w & 3, c0 = (w >> 2) * CPT;
-        const int F = sEA[q * 32 + lane];
+        const int F = eA[q * 32 + lane] - 2112 + P.ash;
         const uint32_t tq = tmem + (uint32_t(q * 32) << 16) + uint32_t(c0);
+        // rolled: the code of one tile has to fit the instruction cache
+        // (unrolled, fetching it cost more than the work)
+#pragma unroll 1
+        for (int cc = 0; cc < CPT; cc += CU) {
+          uint32_t v[kSl][CU];
 #pragma unroll
-        for (int cc = 0; cc < CPT; cc += 4) {
-          uint32_t v[kSl][4];
-#pragma unroll
-          for (int g = 0; g < kSl; ++g) tmem_ld4(tq + uint32_t(g * NT + cc), v[g]);
+          for (int g = 0; g < kSl; ++g) tmem_ld(tq + uint32_t(g * NT + cc), v[g]);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int G = sEB[(c0 + cc + j) >> 1];
-            uint32_t x[kSl];
+          for (int j = 0; j < CU; j += 2) {
+            double d[2];
 #pragma unroll
-            for (int g = 0; g < kSl; ++g) x[g] = v[g][j];
-            double d = join(x, F + G - 2112 + P.ash, P.neg);
-            if (F == 2047 || G == 2047) d = __longlong_as_double(0x7ff8000000000000LL);
-            if (sg == s0) acc[cc + j] = d;
-            else acc[cc + j] += d;
+            for (int i = 0; i < 2; ++i) {
+              float x[kSl];
+#pragma unroll
+              for (int g = 0; g < kSl; ++g) x[g] = __uint_as_float(v[g][j + i]);
+              d[i] = join(x, F + eB[(c0 + cc + j) >> 1], P.neg);
+            }
+            const double2 z = make_double2(d[0], d[1]);
+            if (!P.to_part) *reinterpret_cast<double2*>(stg + cc + j) = z;
+            else if (m < P.M && n0 + ((c0 + cc + j) >> 1) < P.N) prow[(cc + j) >> 1] = z;
           }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       }
-      // sEA / sEB are rewritten by the next segment
-      if (sg + 1 < s1) asm volatile("bar.sync 1, %0;" ::"r"(32 * kWorkers) : "memory");
     }
-    // ---- write the tile, through shared memory so that stores run along C's
-    // contiguous index (the stages are free: every MMA has completed)
-    asm volatile("bar.sync 1, %0;" ::"r"(32 * kWorkers) : "memory");
-    double* stg = reinterpret_cast<double*>(smem);
-    if (ok) {
-      const int q = w & 3, c0 = (w >> 2) * CPT;
+    if (!P.to_part) {
+      // ---- write the tile from shared memory along C's contiguous index
+      asm volatile("bar.sync 1, %0;" ::"r"(32 * kWorkers) : "memory");
+      const double2* sc = reinterpret_cast<const double2*>(smem);
+      constexpr int kEl = kRows * NB / (32 * kWorkers);
+      constexpr int kBatch = kEl % 4 == 0 ? 4 : (kEl % 3 == 0 ? 3 : kEl);
+      static_assert(kEl % kBatch == 0, "store batches");
+#pragma unroll 1
+      for (int e0 = 0; e0 < kEl; e0 += kBatch) {
+        double2 val[kBatch];
+        long long at[kBatch];
 #pragma unroll
-      for (int cc = 0; cc < CPT; cc += 2)
-        *reinterpret_cast<double2*>(&stg[(q * 32 + lane) * (2 * L::kPitch) + c0 + cc]) =
-            make_double2(acc[cc], acc[cc + 1]);
+        for (int u = 0; u < kBatch; ++u) {
+          const int e = (e0 + u) * 32 * kWorkers + tid;
+          const int r = P.c_m ? e % kRows : e / NB, c = P.c_m ? e / kRows : e % NB;
+          const bool in = ok && m0 + r < P.M && n0 + c < P.N;
+          val[u] = sc[r * L::kPitch + c];
+          at[u] = in ? sCM[r] + sCN[c] : -1;
+        }
+        if (P.alpha_rest != 1.0) {
+#pragma unroll
+          for (int u = 0; u < kBatch; ++u) { val[u].x *= P.alpha_rest; val[u].y *= P.alpha_rest; }
+        }
+        if (P.accumulate) {
+          double2 old[kBatch];
+#pragma unroll
+          for (int u = 0; u < kBatch; ++u) old[u] = at[u] >= 0 ? P.C[at[u]] : zero;
+#pragma unroll
+          for (int u = 0; u < kBatch; ++u) { val[u].x += old[u].x; val[u].y += old[u].y; }
+        }
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u)
+          if (at[u] >= 0) P.C[at[u]] = val[u];
+      }
     }
-    asm volatile("bar.sync 1, %0;" ::"r"(32 * kWorkers) : "memory");
-    const double2* sc = reinterpret_cast<const double2*>(smem);
-    constexpr int kEl = kRows * NB / (32 * kWorkers);
-    double2 val[kEl];
-    long long at[kEl];
-#pragma unroll
-    for (int u = 0; u < kEl; ++u) {
-      const int e = u * 32 * kWorkers + int(threadIdx.x);
-      const int r = P.c_m ? e % kRows : e / NB, c = P.c_m ? e / kRows : e % NB;
-      const int m = m0 + r, n = n0 + c;
-      const bool in = ok && m < P.M && n < P.N;
-      val[u] = sc[r * L::kPitch + c];
-      if (P.alpha_rest != 1.0) { val[u].x *= P.alpha_rest; val[u].y *= P.alpha_rest; }
-      at[u] = !in ? -1
-                  : (P.to_part ? ((long long)blockIdx.z * P.M + m) * P.N + n : P.cM[m] + P.cN[n]);
-    }
-    if (P.accumulate) {
-      double2 old[kEl];
-#pragma unroll
-      for (int u = 0; u < kEl; ++u) old[u] = at[u] >= 0 ? P.C[at[u]] : zero;
-#pragma unroll
-      for (int u = 0; u < kEl; ++u) { val[u].x += old[u].x; val[u].y += old[u].y; }
-    }
-#pragma unroll
-    for (int u = 0; u < kEl; ++u)
-      if (at[u] >= 0) P.C[at[u]] = val[u];
   }
   if (!ok && P.err) atomicExch(P.err, 1);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -483,6 +603,39 @@ k_oz_finish(const double2* __restrict__ part, int nsplit, int M, int N, double2*
   C[idx] = v;
 }
 
+// The same for many splits of a small output: a block per four outputs.
+__global__ void __launch_bounds__(512)
+k_oz_finish_wide(const double2* __restrict__ part, int nsplit, int M, int N, double2* __restrict__ C,
+                 const long long* __restrict__ cM, const long long* __restrict__ cN, double alpha,
+                 int accumulate) {
+  __shared__ double2 red[512];
+  const long long total = (long long)M * N;
+  const int o = threadIdx.x & 3;
+  const long long t = (long long)blockIdx.x * 4 + o;
+  double sr = 0.0, si = 0.0;
+  if (t < total) {
+#pragma unroll 8
+    for (int s = threadIdx.x >> 2; s < nsplit; s += 128) {
+      const double2 p = part[(long long)s * total + t];
+      sr += p.x;
+      si += p.y;
+    }
+  }
+  red[threadIdx.x] = make_double2(sr, si);
+  for (int d = 256; d >= 4; d >>= 1) {
+    __syncthreads();
+    if (threadIdx.x < d) {
+      red[threadIdx.x].x += red[threadIdx.x + d].x;
+      red[threadIdx.x].y += red[threadIdx.x + d].y;
+    }
+  }
+  if (threadIdx.x >= 4 || t >= total) return;
+  const long long idx = cM[t / N] + cN[t % N];
+  double2 v = make_double2(alpha * red[o].x, alpha * red[o].y);
+  if (accumulate) { v.x += C[idx].x; v.y += C[idx].y; }
+  C[idx] = v;
+}
+
 template <int NT, bool AKC, bool BKC>
 void launch_nt(const OzArgs& a, dim3 grid, cudaStream_t s) {
   using L = OzSmem<NT>;
@@ -505,7 +658,7 @@ OzPlan oz_plan(long long M, long long N, long long K) {
   const double slots = 152.0;
   for (int sw = 0; sw < 2; ++sw) {
     const long long Mg = sw ? N : M, Ng = sw ? M : N;
-    for (int nt = 64; nt >= 16; nt /= 2) {
+    for (const int nt : {64, 48, 32, 16}) {
       const long long tiles = ((Mg + kRows - 1) / kRows) * ((2 * Ng + nt - 1) / nt);
       // segments: short enough that the tiles fill the GPU, at least 32 k, at
       // most the exactness bound
@@ -514,25 +667,26 @@ OzPlan oz_plan(long long M, long long N, long long K) {
       long long nseg = (K + seg - 1) / seg;
       seg = ((K + nseg - 1) / nseg + 7) / 8 * 8;
       nseg = (K + seg - 1) / seg;
-      // CTAs: one per SM is resident; split the segments while tiles are fewer
-      // than two waves
+      // CTAs: one per SM is resident; with several segments each has its own
+      // partial sum, and a CTA takes several of them in turn once the tiles
+      // fill two waves
       long long zs = std::min(nseg, std::max<long long>(1, (2 * 152) / tiles));
       const long long spc = (nseg + zs - 1) / zs;
       zs = (nseg + spc - 1) / spc;
       // clocks of one segment of one tile: fixed latencies (row maxima,
       // read-back) and 8 complex k at a time, fitted to measurements at
-      // K = 48 .. 1.4e6 with tiles of 32 and 64 columns
-      const double per = double((seg + 7) / 8) * (1900.0 + 18.0 * nt) + 24000.0 + 130.0 * nt;
+      // K = 7 .. 5e6 with every tile width
+      const double per = 14000.0 + double((seg + 7) / 8) * (1500.0 + 8.0 * nt) + 60.0 * nt;
       const double waves = std::ceil(double(tiles * zs) / slots);
-      double cost = waves * double(spc) * per + 4000.0;
-      if (zs > 1) cost += 6000.0 + double(zs) * double(M) * double(N) / slots;
+      double cost = waves * double(spc) * per + 6000.0;
+      if (nseg > 1) cost += 6000.0 + double(nseg) * double(M) * double(N) / slots;
       if (cost < best.cost) {
         best.swap = sw != 0;
         best.nt = nt;
         best.seg = int(seg);
         best.nseg = int(nseg);
         best.spc = int(spc);
-        best.nsplit = int(zs);
+        best.nsplit = int(nseg);
         best.cost = cost;
       }
     }
@@ -572,27 +726,31 @@ int oz_gemm(const OzPlan& p, const OzOperand& A, const OzOperand& B, int M, int 
     const double f = std::frexp(alpha, &e);
     if (std::fabs(f) == 0.5) {
       a.ash = e - 1;
-      a.neg = alpha < 0 ? 1 : 0;
+      a.neg = alpha < 0 ? 0xffffffffu : 0u;
     } else {
       a.alpha_rest = alpha;
     }
   }
   const long long gx = (2LL * N + p.nt - 1) / p.nt, gy = (M + kRows - 1) / kRows;
-  RTCC3_CHECK(gy < 65536 && p.nsplit < 65536, kErrArg, "sliced product: grid too large");
-  dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)p.nsplit);
+  const long long gz = (p.nseg + p.spc - 1) / p.spc;
+  RTCC3_CHECK(gy < 65536 && gz < 65536, kErrArg, "sliced product: grid too large");
+  dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)gz);
 #define RTCC3_OZ(NTV)                                                  \
   if (A.kc && B.kc) launch_nt<NTV, true, true>(a, grid, s);            \
   else if (A.kc) launch_nt<NTV, true, false>(a, grid, s);              \
   else if (B.kc) launch_nt<NTV, false, true>(a, grid, s);              \
   else launch_nt<NTV, false, false>(a, grid, s)
   if (p.nt == 64) { RTCC3_OZ(64); }
+  else if (p.nt == 48) { RTCC3_OZ(48); }
   else if (p.nt == 32) { RTCC3_OZ(32); }
   else { RTCC3_OZ(16); }
 #undef RTCC3_OZ
   if (!split) return 1;
   const long long total = (long long)M * N;
   auto blocks = [&](int po) { return (unsigned)((total + 8LL * po - 1) / (8LL * po)); };
-  if (p.nsplit >= 32)
+  if (p.nsplit >= 256 && total <= 65536)
+    k_oz_finish_wide<<<(unsigned)((total + 3) / 4), 512, 0, s>>>(part, p.nsplit, M, N, C + coff, cM, cN, alpha, accumulate ? 1 : 0);
+  else if (p.nsplit >= 32)
     k_oz_finish<8><<<blocks(4), 256, 0, s>>>(part, p.nsplit, M, N, C + coff, cM, cN, alpha, accumulate ? 1 : 0);
   else
     k_oz_finish<1><<<blocks(32), 256, 0, s>>>(part, p.nsplit, M, N, C + coff, cM, cN, alpha, accumulate ? 1 : 0);
