@@ -130,7 +130,12 @@ KERNEL_FAMILIES = {
     # the two outer products of the X1 / X2 adjoints in one pass
     "k_outer_pair": (("outer_pair",), "hbm"),
     "k_contract": (("contract_simt_c64", "contract_simt_c128"), "alu"),
-    "k_sym6_div": (("sym6_div", "sym3_div"), "hbm"),
+    "k_sym6_orbit": (("sym6_div",), "hbm"),
+    "k_sym3_div": (("sym3_div",), "hbm"),
+    # FP64 products as sliced FP16 tensor-core products
+    "k_oz_gemm": (("contract_sliced_c128",), "tensor"),
+    # small products, a few terms per lane
+    "k_contract_fine": (("contract_fine_c64", "contract_fine_c128"), "alu"),
     "k_pack": (("tc_pack",), "hbm"),
     "k_reduce_small": (("contract_small_c64", "contract_small_c128"), "hbm"),
     "k_gemv": (("contract_gemv_c64", "contract_gemv_c128"), "hbm"),
@@ -144,11 +149,8 @@ KERNEL_FAMILIES = {
 # (kernel, precision, workload) -> bytes.  An entry is removed when its kernel
 # changes after the counters were taken.
 MEASURED_TRAFFIC = {
-    ("k_contract", "tf32", 2): 2.86e6,
     ("k_combine_nd", "tf32", 2): 3.61e6,
     ("k_combine_brick", "tf32", 2): 1755.6e6,
-    ("k_sym6_div", "tf32", 2): 1070.54e6,
-    ("k_reduce_small", "tf32", 2): 149.09e6,
     ("k_tc_gemm", "tf32", 2): 517.74e6,
     ("k_tc_gemm_direct", "tf32", 2): 485.34e6,
     ("k_outer_pair", "tf32", 2): 377.12e6,

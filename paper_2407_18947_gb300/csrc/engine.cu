@@ -136,69 +136,33 @@ __device__ __forceinline__ void brick_coords(int v, unsigned& a, unsigned& b, un
   }
 }
 
-// Y (+)= alpha P(X) / D for X, Y dense (o,o,o,v,v,v): P sums the six
-// simultaneous permutations of (ijk, abc) (NP = 6) or the identity and the
-// exchanges of slot 1 with slots 2 and 3 (NP = 3), then divides by the
-// triples denominator D[ijk abc] = vsum[abc] - osum[ijk] (sums in the compute
-// precision; complex when CPLX).  D is invariant under those permutations, so
-// for NP = 6 the same kernel is its own adjoint.  Grid: ((a, b) bricks,
-// occupied blocks); the occupied blocks are visited in `order` (the distinct
-// permutations of each i <= j <= k consecutively), so the source blocks of
-// one orbit are read while they are resident in L2.
-template <typename R, bool CPLX, int NP>
+// Y (+)= alpha P(X) / D for X, Y dense (o,o,o,v,v,v) with P the sum of the
+// identity and the exchanges of slot 1 with slots 2 and 3 of (ijk, abc),
+// divided by the triples denominator D[ijk abc] = vsum[abc] - osum[ijk] (sums
+// in the compute precision; complex when CPLX).  The occupied blocks are
+// visited in `order` (the distinct permutations of each i <= j <= k
+// consecutively), so the source blocks of one orbit are read while they are
+// resident in L2; consecutive threads are on consecutive abc (two of the
+// three sources keep c fastest).
+template <typename R, bool CPLX>
 __global__ void __launch_bounds__(256)
-k_sym6_div(const Cx<R>* __restrict__ X, Cx<R>* __restrict__ Y, long long offx, long long offy,
+k_sym3_div(const Cx<R>* __restrict__ X, Cx<R>* __restrict__ Y, long long offx, long long offy,
            const R* __restrict__ osum, const R* __restrict__ vsum, const Cx<R>* __restrict__ osum_c,
            const Cx<R>* __restrict__ vsum_c, const int* __restrict__ order, int o, int v, R alpha,
-           int overwrite, const FastDiv fv2, const FastDiv fv, Cx<R>* __restrict__ Y3) {
+           int overwrite, const FastDiv fv2, const FastDiv fv) {
   const int ijk = order ? order[blockIdx.y] : int(blockIdx.y);
   const int i = ijk / (o * o), j = (ijk / o) % o, k = ijk % o;
   const unsigned v2 = unsigned(v) * v, v3 = v2 * v;
   auto O = [&](int x, int y, int z) { return (long long)((x * o + y) * o + z) * v3; };
   const Cx<R>* b0 = X + offx + O(i, j, k);
   const Cx<R>* b1 = X + offx + O(j, i, k);
-  const Cx<R>* b2 = X + offx + O(i, k, j);
   const Cx<R>* b3 = X + offx + O(k, j, i);
-  const Cx<R>* b4 = X + offx + O(k, i, j);
-  const Cx<R>* b5 = X + offx + O(j, k, i);
   Cx<R>* yb = Y + offy + O(i, j, k);
-  // NP = 6 with Y3: also Y3 = (x0 + x1 + x3) / D, the NP = 3 sum of the same
-  // sources (overwritten; dense, no offset)
-  Cx<R>* y3b = Y3 ? Y3 + O(i, j, k) : nullptr;
   auto V = [&](unsigned x, unsigned y, unsigned z) { return (x * v + y) * v + z; };
-  auto element = [&](unsigned a, unsigned b, unsigned c, unsigned abc) {
-    const Cx<R> x0 = b0[abc];
-    const Cx<R> x1 = b1[V(b, a, c)];
-    const Cx<R> x3 = b3[V(c, b, a)];
-    R sr, si;
-    if (NP == 6) {
-      const Cx<R> x2 = b2[V(a, c, b)];
-      const Cx<R> x4 = b4[V(c, a, b)];
-      const Cx<R> x5 = b5[V(b, c, a)];
-      sr = alpha * (((x0.x + x1.x) + (x2.x + x3.x)) + (x4.x + x5.x));
-      si = alpha * (((x0.y + x1.y) + (x2.y + x3.y)) + (x4.y + x5.y));
-      if (y3b) {
-        const R tr = (x0.x + x1.x) + x3.x, ti = (x0.y + x1.y) + x3.y;
-        Cx<R> z;
-        if (CPLX) {
-          const Cx<R> vs = vsum_c[abc], os = osum_c[ijk];
-          const R dr = vs.x - os.x, di = vs.y - os.y;
-          const R m = R(1) / (dr * dr + di * di);
-          const R ir = dr * m, ii = -di * m;
-          z.x = tr * ir - ti * ii;
-          z.y = tr * ii + ti * ir;
-        } else {
-          const R inv = R(1) / (vsum[abc] - osum[ijk]);
-          z.x = tr * inv;
-          z.y = ti * inv;
-        }
-        y3b[abc] = z;
-      }
-    } else {
-      // identity, (ij)(ab) and (ik)(ac): the three slot exchanges with slot 1
-      sr = alpha * ((x0.x + x1.x) + x3.x);
-      si = alpha * ((x0.y + x1.y) + x3.y);
-    }
+  for (unsigned abc = blockIdx.x * blockDim.x + threadIdx.x; abc < v3; abc += gridDim.x * blockDim.x) {
+    const unsigned a = fv2.div(abc), bc = abc - a * v2, b = fv.div(bc), c = bc - b * v;
+    const Cx<R> x0 = b0[abc], x1 = b1[V(b, a, c)], x3 = b3[V(c, b, a)];
+    const R sr = alpha * ((x0.x + x1.x) + x3.x), si = alpha * ((x0.y + x1.y) + x3.y);
     Cx<R> y = overwrite ? cmake<R>(R(0), R(0)) : yb[abc];
     if (CPLX) {
       const Cx<R> vs = vsum_c[abc], os = osum_c[ijk];
@@ -213,23 +177,126 @@ k_sym6_div(const Cx<R>* __restrict__ X, Cx<R>* __restrict__ Y, long long offx, l
       y.y += si * inv;
     }
     yb[abc] = y;
+  }
+}
+
+// Y (+)= alpha P_ijk^abc(X) / D (the six simultaneous permutations of
+// (ijk, abc)) and, WITH3, also Y3 = (X + its slot-1 exchanges) / D, X, Y, Y3
+// dense.  The result is the same at all six permutations of an element and D
+// is invariant, so a CTA takes an 8 x 8 x 8 (a, b, c) brick of one orbit
+// i <= j <= k: it reads the brick's six images (each along its own fastest
+// index, into shared memory), sums and divides once, and writes six images.
+// Every element is read and written once and the arithmetic is a sixth of the
+// element-wise form: at (10, 38), forward and adjoint averaged, 0.52 -> 0.27 ms
+// (complex64: 4 TB/s of HBM traffic) and 3.62 -> 1.17 ms (complex128, bound by
+// the FP64 pipe).  D is invariant, so the kernel is its own adjoint.  Images
+// are stored [x][y][z ^ (x + y)]: rows and columns of any image are at most two
+// to a bank.
+template <typename R, bool CPLX, bool WITH3>
+__global__ void __launch_bounds__(256)
+k_sym6_orbit(const Cx<R>* __restrict__ X, Cx<R>* __restrict__ Y, long long offx, long long offy,
+             const R* __restrict__ osum, const R* __restrict__ vsum,
+             const Cx<R>* __restrict__ osum_c, const Cx<R>* __restrict__ vsum_c, int o, int v, R alpha,
+             int overwrite, Cx<R>* __restrict__ Y3) {
+  // image p holds element (x0, x1, x2) of the orbit's (i, j, k) or (a, b, c) at
+  // (x[P[p][0]], x[P[p][1]], x[P[p][2]])
+  constexpr int P[6][3] = {{0, 1, 2}, {1, 0, 2}, {0, 2, 1}, {2, 1, 0}, {2, 0, 1}, {1, 2, 0}};
+  extern __shared__ __align__(16) unsigned char orbit_smem[];
+  Cx<R>* img = reinterpret_cast<Cx<R>*>(orbit_smem);  // [6][512]
+  Cx<R>* sum = WITH3 ? img + 6 * 512 : img;           // image 0's places otherwise
+  int q = int(blockIdx.y), ijk[3] = {0, 0, 0};
+  while (q >= (o - ijk[0]) * (o - ijk[0] + 1) / 2) { q -= (o - ijk[0]) * (o - ijk[0] + 1) / 2; ++ijk[0]; }
+  ijk[1] = ijk[0];
+  while (q >= o - ijk[1]) { q -= o - ijk[1]; ++ijk[1]; }
+  ijk[2] = ijk[1] + q;
+  const int nb = (v + 7) / 8;
+  const int a0[3] = {int(blockIdx.x) / (nb * nb) * 8, int(blockIdx.x) / nb % nb * 8, int(blockIdx.x) % nb * 8};
+  const unsigned v3 = unsigned(v) * v * v;
+  auto block = [&](int p) {
+    return (long long)((ijk[P[p][0]] * o + ijk[P[p][1]]) * o + ijk[P[p][2]]) * v3;
   };
-  if (NP == 6) {
-    // a CTA covers a 4 (a) x 8 (b) x 8 (c) brick, stepping over c; a warp
-    // covers 2 x 4 x 4 of it, so every source is read in runs of 2 to 4
-    // consecutive elements along its own fastest index (the sources permute
-    // a, b, c)
-    unsigned a, b, c0;
-    brick_coords<1>(v, a, b, c0);
-    if (a >= unsigned(v) || b >= unsigned(v)) return;
-    for (unsigned c = c0; c < unsigned(v); c += 8) element(a, b, c, (a * v + b) * v + c);
-  } else {
-    // two of the three sources keep c fastest: consecutive threads on
-    // consecutive abc
-    for (unsigned abc = blockIdx.x * blockDim.x + threadIdx.x; abc < v3;
-         abc += gridDim.x * blockDim.x) {
-      const unsigned a = fv2.div(abc), bc = abc - a * v2, b = fv.div(bc), c = bc - b * v;
-      element(a, b, c, abc);
+  auto slot = [](int x, int y, int z) { return (x * 8 + y) * 8 + (z ^ ((x + y) & 7)); };
+  const int x = threadIdx.x >> 6, y = (threadIdx.x >> 3) & 7, z = threadIdx.x & 7;  // and x + 4
+  {
+    Cx<R> r[6][2];
+#pragma unroll
+    for (int p = 0; p < 6; ++p) {
+      const Cx<R>* src = X + offx + block(p);
+      const int gy = a0[P[p][1]] + y, gz = a0[P[p][2]] + z;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int gx = a0[P[p][0]] + x + 4 * h;
+        r[p][h] = cmake<R>(R(0), R(0));
+        if (gx < v && gy < v && gz < v) r[p][h] = src[(unsigned(gx) * v + gy) * v + gz];
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < 6; ++p)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) img[p * 512 + slot(x + 4 * h, y, z)] = r[p][h];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int e[3] = {x + 4 * h, y, z};
+    const int a = a0[0] + e[0], b = a0[1] + e[1], c = a0[2] + e[2];
+    if (a >= v || b >= v || c >= v) continue;
+    const unsigned abc = (unsigned(a) * v + b) * v + c;
+    const int block0 = (ijk[0] * o + ijk[1]) * o + ijk[2];
+    R ir, ii = R(0);  // 1 / D
+    if (CPLX) {
+      const Cx<R> vs = vsum_c[abc], os = osum_c[block0];
+      const R dr = vs.x - os.x, di = vs.y - os.y;
+      const R m = R(1) / (dr * dr + di * di);
+      ir = dr * m;
+      ii = -di * m;
+    } else {
+      ir = R(1) / (vsum[abc] - osum[block0]);
+    }
+    auto over = [&](R re, R im) {
+      return CPLX ? cmake<R>(re * ir - im * ii, re * ii + im * ir) : cmake<R>(re * ir, im * ir);
+    };
+    Cx<R> g[6];
+    int at[6];
+#pragma unroll
+    for (int p = 0; p < 6; ++p) {
+      at[p] = p * 512 + slot(e[P[p][0]], e[P[p][1]], e[P[p][2]]);
+      g[p] = img[at[p]];
+    }
+    const Cx<R> s = over(alpha * (((g[0].x + g[1].x) + (g[2].x + g[3].x)) + (g[4].x + g[5].x)),
+                         alpha * (((g[0].y + g[1].y) + (g[2].y + g[3].y)) + (g[4].y + g[5].y)));
+    sum[at[0]] = s;
+    if (WITH3) {
+      // image p: its own element and the images with slots (1, 2) and (1, 3) exchanged
+      constexpr int E12[6] = {1, 0, 4, 5, 2, 3}, E13[6] = {3, 4, 5, 0, 1, 2};
+#pragma unroll
+      for (int p = 0; p < 6; ++p)
+        img[at[p]] = over((g[p].x + g[E12[p]].x) + g[E13[p]].x, (g[p].y + g[E12[p]].y) + g[E13[p]].y);
+    }
+  }
+  __syncthreads();
+  // the distinct blocks of the orbit: two equal occupied indices leave three
+  // images (each element of them once), three equal ones leave one
+  const bool e01 = ijk[0] == ijk[1], e12 = ijk[1] == ijk[2];
+  const unsigned mask = e01 && e12 ? 0x01u : (e01 ? 0x0du : (e12 ? 0x0bu : 0x3fu));
+#pragma unroll
+  for (int p = 0; p < 6; ++p) {
+    if (!(mask >> p & 1)) continue;
+    Cx<R>* dst = Y + offy + block(p);
+    const int gy = a0[P[p][1]] + y, gz = a0[P[p][2]] + z;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int gx = a0[P[p][0]] + x + 4 * h;
+      if (gx >= v || gy >= v || gz >= v) continue;
+      const int t[3] = {x + 4 * h, y, z};
+      int e[3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) e[P[p][d]] = t[d];
+      Cx<R> w = sum[slot(e[0], e[1], e[2])];
+      const unsigned g = (unsigned(gx) * v + gy) * v + gz;
+      if (!overwrite) { w.x += dst[g].x; w.y += dst[g].y; }
+      dst[g] = w;
+      if (WITH3) Y3[block(p) + g] = img[p * 512 + slot(t[0], t[1], t[2])];
     }
   }
 }
@@ -2054,29 +2121,44 @@ void Engine<R>::run_sym6_div(double alpha, const View& X, bool xg, const EpsSpec
   C* py = yg ? nodes_[Y.node].grad : nodes_[Y.node].data;
   const int pk = pbegin();
   const unsigned v2 = unsigned(es.v) * unsigned(es.v), v3 = v2 * unsigned(es.v);
-  const FastDiv fv2(v2), fv(unsigned(es.v));
-  // about four elements per thread along abc; one grid row per occupied block
-  // NP = 6: one CTA per 4 x 8 (a, b) brick of each block; NP = 3: about four
-  // elements per thread along abc
-  dim3 grid(np == 6 ? unsigned((es.v + 3) / 4) * unsigned((es.v + 7) / 8)
-                    : std::max(1u, (v3 + 1023u) / 1024u),
-            unsigned(es.o) * es.o * es.o);
-  RTCC3_CHECK(grid.y < 65536u, kErrArg, "sym6_div: too many occupied blocks");
-#define RTCC3_S6D(CP, NPV)                                                                         \
-  k_sym6_div<R, CP, NPV><<<grid, 256, 0, stream_>>>(px, py, X.off, Y.off, es.osum_r, es.vsum_r,     \
-                                                    es.osum_cr, es.vsum_cr, es.order, es.o, es.v,  \
-                                                    R(alpha), overwrite ? 1 : 0, fv2, fv,    \
-                                                    Y3 ? nodes_[Y3->node].data : nullptr)
-  if (cplx) {
-    if (np == 6) RTCC3_S6D(true, 6);
-    else RTCC3_S6D(true, 3);
+  RTCC3_CHECK(unsigned(es.o) * es.o * es.o < 65536u, kErrArg, "sym6_div: too many occupied blocks");
+  if (np == 6) {
+    const unsigned nb = unsigned(es.v + 7) / 8;
+    const dim3 grid(nb * nb * nb, unsigned(es.o) * (es.o + 1) * (es.o + 2) / 6);
+    const size_t smem = (Y3 ? 7 : 6) * 512 * sizeof(C);
+    C* y3 = Y3 ? nodes_[Y3->node].data : nullptr;
+#define RTCC3_S6O(CP, W3)                                                                          \
+  do {                                                                                             \
+    if (smem > 48 * 1024)                                                                          \
+      RTCC3_CUDA(cudaFuncSetAttribute(k_sym6_orbit<R, CP, W3>,                                     \
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));    \
+    k_sym6_orbit<R, CP, W3><<<grid, 256, smem, stream_>>>(px, py, X.off, Y.off, es.osum_r,         \
+                                                          es.vsum_r, es.osum_cr, es.vsum_cr, es.o, \
+                                                          es.v, R(alpha), overwrite ? 1 : 0, y3);  \
+  } while (0)
+    if (cplx) {
+      if (Y3) RTCC3_S6O(true, true);
+      else RTCC3_S6O(true, false);
+    } else {
+      if (Y3) RTCC3_S6O(false, true);
+      else RTCC3_S6O(false, false);
+    }
+#undef RTCC3_S6O
   } else {
-    if (np == 6) RTCC3_S6D(false, 6);
-    else RTCC3_S6D(false, 3);
+    // about four elements per thread along abc; one grid row per occupied block
+    const FastDiv fv2(v2), fv(unsigned(es.v));
+    const dim3 grid(std::max(1u, (v3 + 1023u) / 1024u), unsigned(es.o) * es.o * es.o);
+    if (cplx)
+      k_sym3_div<R, true><<<grid, 256, 0, stream_>>>(px, py, X.off, Y.off, es.osum_r, es.vsum_r,
+                                                     es.osum_cr, es.vsum_cr, es.order, es.o, es.v,
+                                                     R(alpha), overwrite ? 1 : 0, fv2, fv);
+    else
+      k_sym3_div<R, false><<<grid, 256, 0, stream_>>>(px, py, X.off, Y.off, es.osum_r, es.vsum_r,
+                                                      es.osum_cr, es.vsum_cr, es.order, es.o, es.v,
+                                                      R(alpha), overwrite ? 1 : 0, fv2, fv);
   }
-#undef RTCC3_S6D
   pend(pk, np == 6 ? "sym6_div" : "sym3_div", (np * 2.0 + 8.0) * n,
-       double(n) * sizeof(C) * (np + (overwrite ? 1 : 2)));
+       double(n) * sizeof(C) * (np == 6 ? (overwrite ? 2 : 3) + (Y3 ? 1 : 0) : np + (overwrite ? 1 : 2)));
   ++launches_;
   RTCC3_CUDA(cudaGetLastError());
 }
