@@ -435,9 +435,21 @@ int small_output_config(long long M, long long N) {
   if (M <= 8 && N <= 8) return kSmall8;
   if (M <= 10 && N <= 10) return kSmall10;
   if (M <= 16 && N <= 16) return kSmall16;
+  // 20, 24, 32: the arithmetic goes with the tile's square, so a 20 x 20 output on
+  // the 40 tile did four times its work ((20, 76) occ x occ density, complex64:
+  // 5.8 -> 2.2 ms per slab of two; 27 x 27 on 40: 0.153 -> 0.101 ms).
+  if (M <= 20 && N <= 20) return kSmall20;
+  if (M <= 24 && N <= 24) return kSmall24;
+  if (M <= 32 && N <= 32) return kSmall32;
   if (M <= 40 && N <= 40) return kSmall40;
   if (M <= 48 && N <= 48) return kSmall48;
   if (M <= 64 && N <= 64) return kSmall64;
+  // 76 x 76 on a 2 x 2 grid of 64 x 64 tiles computed 2.8 times its output and read
+  // both operands twice: 12.1 -> 4.9 ms per slab of two of (20, 76).
+  // Tiles of 80 and 96 only where both sides need them: an output of few columns
+  // (M = 95, N = 1) pays for the whole square (0.59 ms instead of 0.02 at 1e6 terms).
+  if (M <= 80 && N <= 80 && N > 40) return kSmall80;
+  if (M <= 96 && N <= 96 && N > 48) return kSmall96;
   if (N == 1 && M <= 256) return kSmallCol256;
   if (N == 1 && M <= 512) return kSmallCol512;
   return kSmallNone;
@@ -449,6 +461,11 @@ double small_output_tile(int cfg) {
     case kSmall8: return 64.0;
     case kSmall10: return 100.0;
     case kSmall16: return 256.0;
+    case kSmall20: return 400.0;
+    case kSmall24: return 576.0;
+    case kSmall32: return 1024.0;
+    case kSmall80: return 6400.0;
+    case kSmall96: return 9216.0;
     case kSmall40: return 1600.0;
     case kSmall48: return 2304.0;
     case kSmall64: return 4096.0;
@@ -465,6 +482,11 @@ int small_output_bk(int cfg, int elem_bytes) {
     case kSmall8: return d ? SmallShape<double, 2, 2, 4, 4>::BK : SmallShape<float, 2, 2, 4, 4>::BK;
     case kSmall10: return d ? SmallShape<double, 2, 2, 5, 5>::BK : SmallShape<float, 2, 2, 5, 5>::BK;
     case kSmall16: return d ? SmallShape<double, 4, 4, 4, 4>::BK : SmallShape<float, 4, 4, 4, 4>::BK;
+    case kSmall20: return d ? SmallShape<double, 4, 4, 5, 5>::BK : SmallShape<float, 4, 4, 5, 5>::BK;
+    case kSmall24: return d ? SmallShape<double, 8, 8, 3, 3>::BK : SmallShape<float, 8, 8, 3, 3>::BK;
+    case kSmall32: return d ? SmallShape<double, 8, 8, 4, 4>::BK : SmallShape<float, 8, 8, 4, 4>::BK;
+    case kSmall80: return d ? SmallShape<double, 16, 16, 5, 5>::BK : SmallShape<float, 16, 16, 5, 5>::BK;
+    case kSmall96: return d ? SmallShape<double, 16, 16, 6, 6>::BK : SmallShape<float, 16, 16, 6, 6>::BK;
     case kSmall40: return d ? SmallShape<double, 8, 8, 5, 5>::BK : SmallShape<float, 8, 8, 5, 5>::BK;
     case kSmall48: return d ? SmallShape<double, 16, 16, 3, 3>::BK : SmallShape<float, 16, 16, 3, 3>::BK;
     case kSmall64: return d ? SmallShape<double, 16, 16, 4, 4>::BK : SmallShape<float, 16, 16, 4, 4>::BK;
@@ -491,6 +513,26 @@ void launch_reduce_small(int cfg, bool a_kc, bool b_kc, const Cx<R>* A, long lon
       break;
     case kSmall10:
       launch_cfg<R, 2, 2, 5, 5>(a_kc, b_kc, A, aoff, aM, aK, B, boff, bN, bK, C, coff, cM, cN, M, N, K,
+                                nsplit, kchunk, alpha, accumulate, part, s);
+      break;
+    case kSmall20:
+      launch_cfg<R, 4, 4, 5, 5>(a_kc, b_kc, A, aoff, aM, aK, B, boff, bN, bK, C, coff, cM, cN, M, N, K,
+                                nsplit, kchunk, alpha, accumulate, part, s);
+      break;
+    case kSmall24:
+      launch_cfg<R, 8, 8, 3, 3>(a_kc, b_kc, A, aoff, aM, aK, B, boff, bN, bK, C, coff, cM, cN, M, N, K,
+                                nsplit, kchunk, alpha, accumulate, part, s);
+      break;
+    case kSmall32:
+      launch_cfg<R, 8, 8, 4, 4>(a_kc, b_kc, A, aoff, aM, aK, B, boff, bN, bK, C, coff, cM, cN, M, N, K,
+                                nsplit, kchunk, alpha, accumulate, part, s);
+      break;
+    case kSmall80:
+      launch_cfg<R, 16, 16, 5, 5>(a_kc, b_kc, A, aoff, aM, aK, B, boff, bN, bK, C, coff, cM, cN, M, N, K,
+                                nsplit, kchunk, alpha, accumulate, part, s);
+      break;
+    case kSmall96:
+      launch_cfg<R, 16, 16, 6, 6>(a_kc, b_kc, A, aoff, aM, aK, B, boff, bN, bK, C, coff, cM, cN, M, N, K,
                                 nsplit, kchunk, alpha, accumulate, part, s);
       break;
     case kSmall40:

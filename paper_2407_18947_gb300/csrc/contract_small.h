@@ -2,7 +2,7 @@
 // 64 x 64 tiled kernel wastes most of its tile and re-reads the long operand.
 //
 //   reduce_small: C[m,n] = sum_k A[m,k] B[n,k] with the whole M x N output held
-//     by every CTA (M, N <= 64, or N = 1 and M <= 512); each CTA sums one K
+//     by every CTA (M, N <= 96, or N = 1 and M <= 512); each CTA sums one K
 //     chunk, so both operands stream from HBM exactly once.  Used for the
 //     triples slot densities (ijkabc,ijkdbc->ad; ijkabc,ljkabc->li) and the
 //     X1-type back-contractions (ijkabc,jkbc->ia).
@@ -20,7 +20,8 @@ namespace rtcc3 {
 // Output-tile configurations of reduce_small (0 = not applicable).
 enum SmallCfg : int {
   kSmallNone = 0, kSmall48 = 1, kSmall16 = 2, kSmallCol256 = 3, kSmallCol512 = 4, kSmall64 = 5,
-  kSmall10 = 6, kSmall40 = 7, kSmall6 = 8, kSmall8 = 9
+  kSmall10 = 6, kSmall40 = 7, kSmall6 = 8, kSmall8 = 9,
+  kSmall20 = 10, kSmall24 = 11, kSmall32 = 12, kSmall80 = 13, kSmall96 = 14
 };
 
 // Configuration for an M x N output (N <= M expected; returns kSmallNone

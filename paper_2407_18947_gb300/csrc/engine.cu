@@ -1247,8 +1247,10 @@ ContractPlan& Engine<R>::plan(const std::string& spec, const View& A, const View
   if (std::is_same<R, double>::value && NB == 1 && K >= 4) {
     const OzPlan oz = oz_plan(M, N, K);
     double terms = double(M) * double(N) * double(K);
-    if (K >= 256 && std::max(M, N) <= 64 && terms > kFineTermsF64)
-      terms = double(K) * small_output_tile(small_output_config(std::max(M, N), std::min(M, N)));
+    const double tile = K >= 256 && std::max(M, N) <= 96 && terms > kFineTermsF64
+                            ? small_output_tile(small_output_config(std::max(M, N), std::min(M, N)))
+                            : 0.0;
+    if (tile > 0.0) terms = double(K) * tile;
     const double simt = 4.0 * terms / (2.0 * 152.0 * 0.85) + 4000.0;
     if (simt > oz.cost) {
       P->use_oz = true;
