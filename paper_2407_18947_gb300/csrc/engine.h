@@ -192,12 +192,14 @@ class Engine {
     cur_tc_ = tc_region_;
     run_contract(spec, alpha, A, ag, B, bg, Cv, cg, accumulate, sa, sb, sc);
   }
-  // Slab of the triples (dense I x o x o x v x v x v, its first occupied
-  // index running over i0 .. i0+I-1): Y = alpha X / D with the triples
-  // denominators D[ijk abc] = vsum[abc] - osum[ijk] of es (the sum tables in
-  // the compute precision, real or complex); X and Y on data buffers, Y may
-  // be X.  Untaped.
-  void exec_slab_div(double alpha, const View& X, int i0, const EpsSpec& es, const View& Y);
+  // Slabs of the triples (dense I x o x o x v x v x v, their first occupied
+  // index running over i0 .. i0+I-1) with the triples denominators
+  // D[ijk abc] = vsum[abc] - osum[ijk] of es (the sum tables in the compute
+  // precision, real or complex), data buffers, untaped, Y none of the sources:
+  // three slabs: Y = alpha (Z1 + Z1(ikjacb) + Z2(ijkbac) + Z2(ikjcab) +
+  // Z3(ikjcba) + Z3(ijkbca)) / D; one slab: Y = alpha (Z1 + Z1(ikjacb)) / D.
+  void exec_slab_sym(double alpha, std::initializer_list<View> zs, int i0, const EpsSpec& es,
+                     const View& Y);
   void exec_axpy(double alpha, const View& X, bool xg, const View& Y, bool yg) {
     run_axpy(alpha, X, xg, Y, yg);
   }

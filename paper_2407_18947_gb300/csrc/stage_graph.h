@@ -158,7 +158,7 @@ void blocked_triples(Engine<R>& E, int o, int v, int chunk, const TriplesOperand
   // occupied position, Z1[i,j,k,..] = Z[i,j,k,..], Z2[i,j,k,..] = Z[j,i,k,..]
   // and Z3[i,j,k,..] = Z[j,k,i,..] (two products each), then
   // W = Z1 + Z1(ikjacb) + Z2(ijkbac) + Z2(ikjcab) + Z3(ikjcba) + Z3(ijkbca)
-  // (the six terms of P_ijk^abc) in one pass, and t3 = -W / D.
+  // (the six terms of P_ijk^abc) and t3 = -W / D in one pass.
   auto build_t3 = [&E, prod, in, es](const View& T, const View& Z1, const View& Z2, const View& Z3,
                                      int i0, int I) {
     const View* Zs[3] = {&Z1, &Z2, &Z3};
@@ -170,11 +170,7 @@ void blocked_triples(Engine<R>& E, int o, int v, int chunk, const TriplesOperand
       prod(kB[p], -1.0, {in.T2, false, false}, {in.G2, false, false}, {*Zs[p], false, true}, i0, I,
            true);
     }
-    E.exec_combine({{1.0, Z1}, {1.0, E.ev("ikjacb->ijkabc", Z1)}, {1.0, E.ev("ijkbac->ijkabc", Z2)},
-                    {1.0, E.ev("ikjcab->ijkabc", Z2)}, {1.0, E.ev("ikjcba->ijkabc", Z3)},
-                    {1.0, E.ev("ijkbca->ijkabc", Z3)}},
-                   T, true);
-    E.exec_slab_div(-1.0, T, i0, es, T);
+    E.exec_slab_sym(-1.0, {Z1, Z2, Z3}, i0, es, T);
   };
   const View X1v = E.v(X1o), S3v = E.v(S3o);
   for (int i0 = 0; i0 < o; i0 += I0) {
@@ -256,8 +252,7 @@ void blocked_triples(Engine<R>& E, int o, int v, int chunk, const TriplesOperand
                I, !first);
           first = false;
         }
-      E.exec_combine({{1.0, U}, {1.0, E.ev("ikjacb->ijkabc", U)}}, W, true);
-      E.exec_slab_div(1.0, W, i0, es, W);  // W = P(Q) / D = -grad Z
+      E.exec_slab_sym(1.0, {U}, i0, es, W);  // W = P(Q) / D = -grad Z
       if (gfield) {
         // slot densities of the symmetrised y' = P(Q) / (6 D) with t3,
         // summed over the three slots: 1/2 of one slot of P(Q) / D
