@@ -1435,27 +1435,32 @@ ContractPlan& Engine<R>::plan(const std::string& spec, const View& A, const View
   // equations to converge.
   const long long kp_tc = tc_ok ? 2LL * tc_packed_k(int(K), 4) : 0;
   const bool long_k = K >= 64 && M * N * K >= (1LL << 21);
-  const bool out_bound = tc_eb_ == 4 && M * N >= (1LL << 22) && M * N >= 2 * (M + 2 * N) * kp_tc;
+  // (a sum of up to six K tiles: its operand's parts fit tensor memory; above
+  // 64 complex terms, where the alternative packs both operands too, the line
+  // lies where the packed operands are as large as the output)
+  const bool c_unit_m = !gm.empty() && std::llabs(gm.back().sc) == 1;
+  const bool out_bound =
+      tc_eb_ == 4 && M * N >= (1LL << 22) && kp_tc <= 64 * kTcShortKb &&
+      (long_k ? 2 * M * N >= kp_tc * (c_unit_m ? M + 4 * N : N + 4 * M) : M * N >= 2 * (M + 2 * N) * kp_tc);
   if (std::is_same<R, float>::value && tc_ok && NB == 1 && std::max(M, N) >= 128 &&
       std::min(M, N) >= 4 && (long_k || out_bound)) {
     P->use_tc = true;
     // long sums: the expanded (2x2 real) operand is the smaller one; short
-    // sums: the output's contiguous index goes to the GEMM columns, which
-    // the epilogue stores in runs
-    const bool c_unit_m = !gm.empty() && std::llabs(gm.back().sc) == 1;
-    P->tc_swap = long_k ? (N > M) : c_unit_m;
-    P->tc_out = !long_k;
+    // sums: the output's contiguous index goes to the GEMM rows, which are the
+    // lanes of the accumulator, so a warp stores it in runs
+    P->tc_out = out_bound;
+    P->tc_swap = out_bound ? !c_unit_m : N > M;
     const long long Mg = P->tc_swap ? N : M, Ng = P->tc_swap ? M : N;
     P->tc_kp = tc_packed_k(int(K), tc_eb_);
     const int nkb = P->tc_kp / (128 / tc_eb_);
     const long long nr = 2 * Ng;
-    const long long bn = tc_tile_n(int(std::min<long long>(nr, 1 << 30)), P->tc_out);
+    const long long bn = tc_tile_n(int(std::min<long long>(nr, 1 << 30)));
     const long long tcs = ((nr + bn - 1) / bn) * ((Mg + 127) / 128);
     // split K so that the CTAs fill whole waves of the GPU (each split sums
     // at least 32 K tiles; a larger split must gain 3% of wave occupancy)
     int ts = 1;
     if (!P->tc_out && nkb >= 64) {
-      const long long slots = 152LL * tc_ctas_per_sm(false);
+      const long long slots = 152LL;
       double best = double(tcs) / double(((tcs + slots - 1) / slots) * slots);
       for (int c = 2; c <= nkb / 32 && c <= 64; ++c) {
         const long long ctas = tcs * c;

@@ -68,7 +68,7 @@ struct ContractPlan {
   // tensor-core route (complex64 graphs with TF32/BF16 operands)
   bool use_tc = false, tc_swap = false;
   int tc_nsplit = 1, tc_kp = 0;
-  bool tc_out = false;  // short sum bound by its output (two CTAs per SM)
+  bool tc_out = false;  // short sum bound by its output (k_tc_gemm_short)
   // small products spread over the GPU, a few terms per lane (FineArgs)
   bool use_fine = false, fine_block = false;
   int fine_ls = 0;

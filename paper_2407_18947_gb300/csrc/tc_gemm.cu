@@ -8,8 +8,9 @@
 // memory (the MMA warp then issues hi.hi, hi.lo and lo.hi) and afterwards
 // read the FP32 accumulator back with tcgen05.ld and write the complex result
 // (coalesced through a per-warp shared-memory transpose, 16 stores in flight
-// per warp) or FP32 split-K partials.  Used for the short sums bound by their
-// output.
+// per warp) or FP32 split-K partials.
+//
+// k_tc_gemm_short: short TF32 sums bound by their output, persistent.
 //
 // k_tc_gemm_direct (TF32 long sums) and k_tc_gemm_chains (BF16 long sums)
 // cut the sum into accumulation chains and let one CTA stream several chains
@@ -154,12 +155,11 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
 
 // Shared-memory plan of one CTA.  SPLIT (TF32 with a hi + lo split done in
 // shared memory): A arrives as raw FP32 and a second A buffer takes the low
-// parts; B arrives pre-split as [hi | lo] K halves.  EW epilogue warps: 8
-// with a ring of up to four stages in 192 KB (one CTA per SM, long sums), or
-// 4 with the ring in 80 KB (two CTAs per SM: one CTA's epilogue overlaps the
-// other's main loop, for products bound by their output).
-template <int BN, bool SPLIT, int EW>
+// parts; B arrives pre-split as [hi | lo] K halves.  A ring of up to four
+// stages in 192 KB, one CTA per SM.
+template <int BN, bool SPLIT>
 struct TcSmem {
+  static constexpr int EW = 8;  // epilogue warps
   // TMEM columns of the FP32 accumulator (an allocation is a power of two >= 32)
   static constexpr int kTmemCols = BN <= 32 ? 32 : (BN <= 64 ? 64 : (BN <= 128 ? 128 : 256));
   static constexpr int kABytes = kBM * 128;
@@ -168,7 +168,7 @@ struct TcSmem {
   static constexpr int kBLoBytes = SPLIT ? BN * 128 : 0;
   static constexpr int kStageBytes = kABytes + kALoBytes + kBBytes + kBLoBytes;
   static constexpr int kTmaBytes = kABytes + kBBytes + kBLoBytes;  // bytes the TMA delivers
-  static constexpr int kRing = EW == 8 ? 196608 : 81920;
+  static constexpr int kRing = 196608;
   static constexpr int kStages = kRing / kStageBytes < 4 ? kRing / kStageBytes : 4;
   static constexpr int kBarOff = kStages * kStageBytes;
   static constexpr int kStageOutOff = kBarOff + 256;
@@ -176,17 +176,18 @@ struct TcSmem {
   static constexpr int kTotal = kStageOutOff + kStageOutBytes + 1024;  // + alignment slack
   static constexpr int kThreads = 64 + 32 * EW;  // TMA warp, MMA warp, EW epilogue warps
   static_assert(kStages >= 1, "ring depth");
-  static_assert(kTotal <= (EW == 8 ? 232448 : 116224), "shared memory per CTA");
+  static_assert(kTotal <= 232448, "shared memory per CTA");
 };
 
-template <int BN, bool BF16, bool SPLIT, int EW>
-__global__ void __launch_bounds__(64 + 32 * EW, EW == 4 ? 2 : 1)
+template <int BN, bool BF16, bool SPLIT>
+__global__ void __launch_bounds__(320, 1)
 k_tc_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
           int M, int Nr, int nkb_total, int kb_per_split, int kb_lo, float2* __restrict__ C,
           const long long* __restrict__ cM, const long long* __restrict__ cN, long long coff,
           float alpha, int accumulate, float* __restrict__ partial, int* __restrict__ err,
           long long budget) {
-  using L = TcSmem<BN, SPLIT, EW>;
+  using L = TcSmem<BN, SPLIT>;
+  constexpr int EW = L::EW;
   constexpr int kStages = L::kStages;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -611,6 +612,315 @@ k_tc_gemm_chains(const uint8_t* __restrict__ Atiled, const __grid_constant__ CUt
   }
 }
 
+// Short TF32 sums (at most kTcShortKb K tiles) with a large output: the
+// connected triples and their cotangents.  One persistent CTA per SM keeps a
+// row block's A, split once into hi and lo, in tensor memory for the whole sum
+// (64 columns per K tile) and streams the column tiles of B ([hi | lo]) past
+// it through a ring, so loads, MMAs and stores of successive tiles overlap;
+// two 128-column accumulators where tensor memory has room (four K tiles), one
+// beyond (its drain costs about a tenth).  The output's contiguous index is on
+// the rows, that is on the accumulator's lanes: a warp stores 256-byte runs
+// straight from its registers.
+//
+// As one CTA per 128 x 128 tile with a single load - split - MMA stage, each
+// tile pair took 44,000 cycles of mostly latency.  Complex64 times, before ->
+// now: 2432 x 92416 x 92 1.9 -> 0.69 ms (241 TFLOP/s, 722 with the three split
+// products, 65 % of the TF32 rate: bound by the MMAs and the reads of B from
+// L2); 3800 x 14440 x 48 0.18 -> 0.098 ms; accumulating 92416 x 2432 x 16 1.55
+// -> 0.85 ms (4.3 TB/s of read and written output).  64-column tiles run the
+// tensor pipe at half rate (0.163 instead of 0.097 ms at 3800 x 14440 x 48).
+//
+// Shared memory: the ring of B stages (128 rows of one K tile, hi and lo), two
+// raw A tiles on their way into tensor memory and, when accumulating, the
+// prefetched output tile.
+template <int NACC, bool ACC>
+struct TcShortSmem {
+  static constexpr int BN = 128;
+  static constexpr int kABytes = kBM * 128;
+  static constexpr int kStage = 2 * BN * 128;
+  static constexpr int kOldBytes = ACC ? kBM * (BN / 2) * 8 : 0;  // prefetched output tile
+  static constexpr int kStages = (232448 - 1024 - 512 - 2 * kABytes - kOldBytes) / kStage;
+  static constexpr int kACol = NACC * BN;
+  static constexpr int kMaxKb = (512 - kACol) / 64;
+  static constexpr int kAOff = kStages * kStage;
+  static constexpr int kOldOff = kAOff + 2 * kABytes;
+  static constexpr int kBarOff = kOldOff + kOldBytes;
+  static constexpr int kTotal = kBarOff + 512 + 1024;  // barriers + alignment slack
+  static_assert(kStages >= 2 && kTotal <= 232448, "plan");
+};
+
+template <int NACC, bool ACC>
+__global__ void __launch_bounds__(608, 1)
+k_tc_gemm_short(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                int M, int N, int nkb, int mblocks, int nblocks, int tpc, int units,
+                float2* __restrict__ C, const long long* __restrict__ cM,
+                const long long* __restrict__ cN, long long coff, float alpha,
+                int* __restrict__ err, long long budget) {
+  using L = TcShortSmem<NACC, ACC>;
+  constexpr int S = L::kStages, BN = L::BN;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::kBarOff);
+  uint64_t* full = bars;                // [S] B stage landed
+  uint64_t* empty = full + S;           // [S] its MMAs done (commit)
+  uint64_t* afull = empty + S;          // [2] raw A tile landed
+  uint64_t* aempty = afull + 2;         // [2] raw A tile split (4 warps)
+  uint64_t* aconv = aempty + 2;         // [kMaxKb] K tile of A in tensor memory (4 warps)
+  uint64_t* cfull = aconv + L::kMaxKb;  // [2] accumulator holds a finished tile
+  uint64_t* cfree = cfull + 2;          // [2] accumulator read (16 warps)
+  uint64_t* udone = cfree + 2;          // MMAs of a row block done: A may be replaced
+  uint64_t* fin = udone + 1;            // every MMA issued has completed
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fin + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < S; ++s) {
+      mbar_init(smem_u32(&full[s]), 1);
+      mbar_init(smem_u32(&empty[s]), 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(smem_u32(&afull[b]), 1);
+      mbar_init(smem_u32(&aempty[b]), 4);
+      mbar_init(smem_u32(&cfull[b]), 1);
+      mbar_init(smem_u32(&cfree[b]), 16);
+    }
+    for (int k = 0; k < L::kMaxKb; ++k) mbar_init(smem_u32(&aconv[k]), 4);
+    mbar_init(smem_u32(udone), 1);
+    mbar_init(smem_u32(fin), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(512)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tmem_slot;
+  bool ok = true;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int it = 0, s = 0, ph = 1;  // ph: parity of the stage's previous release
+      for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+        const int t0 = u / mblocks * tpc, t1 = min(nblocks, t0 + tpc);
+        for (int t = t0; t < t1 && ok; ++t)
+          for (int kb = 0; kb < nkb; ++kb) {
+            if (it >= S) ok = mbar_wait(smem_u32(&empty[s]), ph, budget);
+            if (!ok) break;
+            const uint32_t fb = smem_u32(&full[s]);
+            const uint32_t sb = smem_u32(smem + s * L::kStage);
+            mbar_expect_tx(fb, L::kStage);
+            tma_load_2d(sb, &tmB, kb * 32, t * BN, fb);
+            tma_load_2d(sb + BN * 128, &tmB, (kb + nkb) * 32, t * BN, fb);
+            ++it;
+            if (++s == S) { s = 0; ph ^= 1; }
+          }
+      }
+      // no copy into shared memory may be outstanding at exit (also after
+      // giving up): the last ring round of copies has landed
+      for (int i = max(0, it - S); i < it; ++i)
+        if (!mbar_wait(smem_u32(&full[i % S]), (i / S) & 1, kDrainBudget)) ok = false;
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      constexpr uint32_t idesc = instr_desc<false>(kBM, BN);
+      int s = 0, ph = 0, j = 0, ui = 0;
+      for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++ui) {
+        const int t0 = u / mblocks * tpc, t1 = min(nblocks, t0 + tpc);
+        for (int t = t0; t < t1 && ok; ++t, ++j) {
+          const int b = j % NACC;
+          if (j >= NACC) ok = mbar_wait(smem_u32(&cfree[b]), (j / NACC - 1) & 1, budget);
+          const uint32_t acc_t = tmem + uint32_t(b * BN);
+          for (int kb = 0; kb < nkb && ok; ++kb) {
+            if (t == t0) ok = mbar_wait(smem_u32(&aconv[kb]), ui & 1, budget);
+            ok = ok && mbar_wait(smem_u32(&full[s]), ph, budget);
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t sb = smem_u32(smem + s * L::kStage);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+              const uint32_t ah = tmem + uint32_t(L::kACol + 64 * kb + 8 * kk);
+              mma_tf32_ta(acc_t, ah, smem_desc(sb + kk * 32), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+              mma_tf32_ta(acc_t, ah, smem_desc(sb + BN * 128 + kk * 32), idesc, 1u);
+              mma_tf32_ta(acc_t, ah + 32, smem_desc(sb + kk * 32), idesc, 1u);
+            }
+            mma_commit(smem_u32(&empty[s]));
+            if (++s == S) { s = 0; ph ^= 1; }
+          }
+          if (ok) mma_commit(smem_u32(&cfull[b]));
+        }
+        if (ok) mma_commit(smem_u32(udone));
+      }
+      // every MMA issued has completed before tensor memory is freed (also
+      // after giving up)
+      mma_commit(smem_u32(fin));
+      if (!mbar_wait(smem_u32(fin), 0, kDrainBudget)) ok = false;
+    }
+  } else if (warp == 2) {
+    if (lane == 0) {
+      int ia = 0;
+      for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+        const int m0 = u % mblocks * kBM;
+        for (int kb = 0; kb < nkb; ++kb) {
+          const int b = ia & 1;
+          if (ia >= 2) ok = mbar_wait(smem_u32(&aempty[b]), ((ia >> 1) - 1) & 1, budget);
+          if (!ok) break;
+          const uint32_t fb = smem_u32(&afull[b]);
+          mbar_expect_tx(fb, L::kABytes);
+          tma_load_2d(smem_u32(smem + L::kAOff + b * L::kABytes), &tmA, kb * 32, m0, fb);
+          ++ia;
+        }
+      }
+      for (int i = max(0, ia - 2); i < ia; ++i)
+        if (!mbar_wait(smem_u32(&afull[i & 1]), (i >> 1) & 1, kDrainBudget)) ok = false;
+    }
+  } else {
+    // warps 3-18: TMEM lane quarter warp % 4, 32-column chunk e / 4
+    const int e = warp - 3, chunk = e >> 2, q = warp & 3;
+    const uint32_t lane_base = uint32_t(32 * q) << 16;
+    const int row = 32 * q + lane;
+    float2* oldp = reinterpret_cast<float2*>(smem + L::kOldOff) + (threadIdx.x - 96);
+    const uint32_t old = smem_u32(oldp);
+    int j = 0, ia = 0, ui = 0;
+    for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++ui) {
+      const int m = u % mblocks * kBM + row;
+      const int t0 = u / mblocks * tpc, t1 = min(nblocks, t0 + tpc);
+      if (e < 4) {
+        // split the row block's A into hi and lo in tensor memory once the
+        // MMAs of the previous row block are done with it
+        if (ui > 0) ok = mbar_wait(smem_u32(udone), (ui - 1) & 1, budget);
+        ok = __all_sync(0xffffffffu, ok);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        for (int kb = 0; kb < nkb && ok; ++kb, ++ia) {
+          ok = mbar_wait(smem_u32(&afull[ia & 1]), (ia >> 1) & 1, budget);
+          ok = __all_sync(0xffffffffu, ok);  // tcgen05.st below is warp-collective
+          if (!ok) break;
+          const float4* ar = reinterpret_cast<const float4*>(smem + L::kAOff + (ia & 1) * L::kABytes + row * 128);
+          uint32_t hi[32], lo[32];
+#pragma unroll
+          for (int c = 0; c < 8; ++c) {
+            const float4 x = ar[c ^ (row & 7)];
+            const float xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+            for (int d = 0; d < 4; ++d) {
+              hi[4 * c + d] = to_tf32(xv[d]);
+              lo[4 * c + d] = __float_as_uint(xv[d] - __uint_as_float(hi[4 * c + d]));
+            }
+          }
+          const uint32_t ta = tmem + lane_base + uint32_t(L::kACol + 64 * kb);
+          tmem_st32(ta, hi);
+          tmem_st32(ta + 32, lo);
+          asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) {
+            mbar_arrive(smem_u32(&aempty[ia & 1]));
+            mbar_arrive(smem_u32(&aconv[kb]));
+          }
+        }
+      }
+      const bool rin = m < M;
+      float2* crow = C + (coff + (rin ? cM[m] : 0));
+      // ACC: the output tile's old values come by asynchronous copies into this
+      // thread's own places, one tile ahead of the MMAs
+      auto prefetch = [&](int t) {
+        const int n0 = t * (BN / 2) + 16 * chunk, nc = rin ? min(16, N - n0) : 0;
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+          if (k < nc) cp_async8(old + k * 4096, crow + __ldg(cN + n0 + k), 8u);
+      };
+      if (ACC) prefetch(t0);
+      for (int t = t0; t < t1 && ok; ++t, ++j) {
+        const int b = j % NACC;
+        ok = mbar_wait(smem_u32(&cfull[b]), (j / NACC) & 1, budget);
+        ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld below is warp-collective
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        uint32_t r[32];
+        tmem_ld32(tmem + lane_base + uint32_t(b * BN + 32 * chunk), r);
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&cfree[b]));
+        float2 v[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+          v[k] = make_float2(alpha * __uint_as_float(r[2 * k]), alpha * __uint_as_float(r[2 * k + 1]));
+        if (ACC) {
+          asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll
+          for (int k = 0; k < 16; ++k) {
+            const float2 w = oldp[k * 512];
+            v[k].x += w.x;
+            v[k].y += w.y;
+          }
+          if (t + 1 < t1) prefetch(t + 1);
+        }
+        const int n0 = t * (BN / 2) + 16 * chunk, nc = rin ? min(16, N - n0) : 0;
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+          if (k < nc) crow[__ldg(cN + n0 + k)] = v[k];
+      }
+    }
+    // no copy may be outstanding at exit
+    if (ACC) asm volatile("cp.async.wait_all;" ::: "memory");
+  }
+  if (!ok && err) atomicExch(err, 1);
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 1) {
+    __syncwarp();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512)
+                 : "memory");
+  }
+}
+
+// Units of one row block and a run of column tiles, row blocks fastest so that
+// the CTAs of a wave read the same columns of B; the runs as long as a balanced
+// number of waves allows (a change of row block costs about two tiles).
+template <int NACC>
+void launch_short(const CUtensorMap& ma, const CUtensorMap& mb, const TcOperands& op, float2* C,
+                  const long long* cM, const long long* cN, long long coff, float alpha,
+                  bool accumulate, int* err, cudaStream_t s) {
+  constexpr int BN = TcShortSmem<NACC, true>::BN;
+  static bool attr = false;
+  if (!attr) {
+    RTCC3_CUDA(cudaFuncSetAttribute(k_tc_gemm_short<NACC, true>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    TcShortSmem<NACC, true>::kTotal));
+    RTCC3_CUDA(cudaFuncSetAttribute(k_tc_gemm_short<NACC, false>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    TcShortSmem<NACC, false>::kTotal));
+    attr = true;
+  }
+  const int nkb = op.Kp / 32, mblocks = (op.M + kBM - 1) / kBM, nblocks = (2 * op.N + BN - 1) / BN;
+  long long best = -1;
+  int tpc = nblocks;
+  for (int z = 1; z <= nblocks && z <= 304; ++z) {
+    const int per = (nblocks + z - 1) / z;
+    const long long units = (long long)mblocks * ((nblocks + per - 1) / per);
+    const long long cost = (units + 151) / 152 * (per + 2);
+    if (best < 0 || cost < best) {
+      best = cost;
+      tpc = per;
+    }
+  }
+  const int units = mblocks * ((nblocks + tpc - 1) / tpc);
+  const long long budget = op.wait_budget > 0 ? op.wait_budget : kWaitBudget;
+  const int grid = std::min(units, 152);
+  if (accumulate)
+    k_tc_gemm_short<NACC, true><<<grid, 608, TcShortSmem<NACC, true>::kTotal, s>>>(
+        ma, mb, op.M, op.N, nkb, mblocks, nblocks, tpc, units, C, cM, cN, coff, alpha, err, budget);
+  else
+    k_tc_gemm_short<NACC, false><<<grid, 608, TcShortSmem<NACC, false>::kTotal, s>>>(
+        ma, mb, op.M, op.N, nkb, mblocks, nblocks, tpc, units, C, cM, cN, coff, alpha, err, budget);
+  RTCC3_CUDA(cudaGetLastError());
+}
+
 // One thread per complex source element: its (re, im) pair is written to
 // every K segment (and, for B, to both rows of its 2x2 embedding) with one
 // vector store each.  I is the index type of the flattened (row, k) loop.
@@ -759,14 +1069,14 @@ bool make_map(CUtensorMap* map, const void* base, int elem_bytes, int Kp, int ro
   return r == CUDA_SUCCESS;
 }
 
-template <int BN, bool BF16, bool SPLIT, int EW>
+template <int BN, bool BF16, bool SPLIT>
 void launch(const CUtensorMap& ma, const CUtensorMap& mb, const TcOperands& op, float2* C,
             const long long* cM, const long long* cN, long long coff, float alpha, bool accumulate,
             int nsplit, float* partial, int* err, cudaStream_t s) {
-  using L = TcSmem<BN, SPLIT, EW>;
+  using L = TcSmem<BN, SPLIT>;
   static bool attr = false;
   if (!attr) {
-    RTCC3_CUDA(cudaFuncSetAttribute(k_tc_gemm<BN, BF16, SPLIT, EW>,
+    RTCC3_CUDA(cudaFuncSetAttribute(k_tc_gemm<BN, BF16, SPLIT>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal));
     attr = true;
   }
@@ -774,7 +1084,7 @@ void launch(const CUtensorMap& ma, const CUtensorMap& mb, const TcOperands& op, 
   const int nkb = op.Kp / (128 / op.elem_bytes);
   const int per = (nkb + nsplit - 1) / nsplit;
   dim3 grid((Nr + BN - 1) / BN, (op.M + kBM - 1) / kBM, nsplit);
-  k_tc_gemm<BN, BF16, SPLIT, EW><<<grid, L::kThreads, L::kTotal, s>>>(
+  k_tc_gemm<BN, BF16, SPLIT><<<grid, L::kThreads, L::kTotal, s>>>(
       ma, mb, op.M, Nr, nkb, per, nkb, C, cM, cN, coff, alpha, accumulate ? 1 : 0,
       nsplit > 1 ? partial : nullptr, err, op.wait_budget > 0 ? op.wait_budget : kWaitBudget);
   RTCC3_CUDA(cudaGetLastError());
@@ -1260,15 +1570,15 @@ bool tc_gemm(const void* Apack, const void* Bpack, const TcOperands& op, float2*
   const int Nr = 2 * op.N;
   if (op.M <= 0 || op.N <= 0 || op.Kp <= 0) return false;
   if (op.Kp % (128 / op.elem_bytes) != 0) return false;
-  const int BN = tc_tile_n(Nr, op.out_bound);
+  const int BN = op.out_bound ? 128 : tc_tile_n(Nr);
   CUtensorMap ma, mb;
   if (!op.a_tiled && !make_map(&ma, Apack, op.elem_bytes, op.Kp, op.M, kBM)) return false;
   if (!make_map(&mb, Bpack, op.elem_bytes, op.split ? 2 * op.Kp : op.Kp, Nr, BN)) return false;
   const bool bf16 = op.elem_bytes == 2;
   RTCC3_CHECK(bf16 || op.split, kErrArg, "TF32 operands are split in the GEMM (pack B as hi | lo)");
-#define RTCC3_TC(BNV, EWV)                                                                        \
-  (bf16 ? launch<BNV, true, false, EWV>(ma, mb, op, C, cM, cN, coff, alpha, accumulate, nsplit, partial, err_flag, s) \
-        : launch<BNV, false, true, EWV>(ma, mb, op, C, cM, cN, coff, alpha, accumulate, nsplit, partial, err_flag, s))
+#define RTCC3_TC(BNV)                                                                        \
+  (bf16 ? launch<BNV, true, false>(ma, mb, op, C, cM, cN, coff, alpha, accumulate, nsplit, partial, err_flag, s) \
+        : launch<BNV, false, true>(ma, mb, op, C, cM, cN, coff, alpha, accumulate, nsplit, partial, err_flag, s))
 #define RTCC3_CH(BNV)                                                                     \
   (bf16 ? launch_chains<BNV, true, false>(Apack, mb, op, nsplit, partial, err_flag, s)     \
         : launch_chains<BNV, false, true>(Apack, mb, op, nsplit, partial, err_flag, s))
@@ -1282,14 +1592,15 @@ bool tc_gemm(const void* Apack, const void* Bpack, const TcOperands& op, float2*
     else if (BN == 32) launched = RTCC3_CH(32);
     RTCC3_CHECK(launched, kErrArg, "chained long sum: unsupported tile");
   } else if (op.out_bound) {
-    if (BN == 128) RTCC3_TC(128, 4);
-    else RTCC3_TC(64, 4);
+    RTCC3_CHECK(op.split && nsplit == 1 && op.Kp <= 32 * kTcShortKb, kErrArg, "output-bound products are unsplit TF32 sums");
+    if (op.Kp <= 128) launch_short<2>(ma, mb, op, C, cM, cN, coff, alpha, accumulate, err_flag, s);
+    else launch_short<1>(ma, mb, op, C, cM, cN, coff, alpha, accumulate, err_flag, s);
   } else {
-    if (BN == 256) RTCC3_TC(256, 8);
-    else if (BN == 128) RTCC3_TC(128, 8);
-    else if (BN == 96) RTCC3_TC(96, 8);
-    else if (BN == 64) RTCC3_TC(64, 8);
-    else RTCC3_TC(32, 8);
+    if (BN == 256) RTCC3_TC(256);
+    else if (BN == 128) RTCC3_TC(128);
+    else if (BN == 96) RTCC3_TC(96);
+    else if (BN == 64) RTCC3_TC(64);
+    else RTCC3_TC(32);
   }
 #undef RTCC3_TC
 #undef RTCC3_CH
@@ -1301,7 +1612,7 @@ bool tc_gemm_direct(const float2* A, long long aoff, const long long* aM, const 
                     int* err_flag, cudaStream_t s) {
   RTCC3_CHECK(tc_direct(op, nsplit) && partial, kErrArg, "direct long sum: unsupported shape");
   const int Nr = 2 * op.N;
-  const int BN = tc_tile_n(Nr, false);
+  const int BN = tc_tile_n(Nr);
   CUtensorMap mb;
   if (!make_map(&mb, Bpack, 4, 2 * op.Kp, Nr, BN)) return false;
   if (BN == 128) launch_direct<128>(A, aoff, aM, aK, a_kc, mb, op, nsplit, partial, err_flag, s);

@@ -25,8 +25,9 @@ struct TcOperands {
   // sums hi.hi + hi.lo + lo.hi (FP32-level products at three times the
   // tensor work, A read once).
   bool split = false;
-  // the product is bound by its output (short sum): two CTAs per SM with
-  // narrower tiles, so that epilogues overlap main loops
+  // the product is bound by its output (TF32 split, a sum of at most
+  // kTcShortKb K tiles): k_tc_gemm_short; the output's contiguous index is
+  // that of the rows
   bool out_bound = false;
   // A packed in tiles of 128 rows x 128 bytes of K, each stored as the
   // 128-byte-swizzled shared-memory image the MMA reads and the tiles of one
@@ -39,11 +40,12 @@ struct TcOperands {
   long long wait_budget = 0;
 };
 
+// K tiles (32 real K each) whose A parts fit tensor memory beside a 128-column
+// accumulator.
+constexpr int kTcShortKb = 6;
 // GEMM column tile (real columns) for Nr = 2N real output columns: the
-// narrowest of 64 / 128 / 256 that holds them (one column tile, the A tile
-// read once), at most 128 for output-bound products.
-inline int tc_tile_n(int Nr, bool out_bound) {
-  if (out_bound) return Nr <= 64 ? 64 : 128;
+// narrowest that holds them (one column tile, the A tile read once).
+inline int tc_tile_n(int Nr) {
   // long sums with narrow outputs: the tile's unused columns are tensor-core
   // work the operand stream has to wait for (N = 10 complex -> 20 real
   // columns, N = 38 -> 76)
@@ -53,14 +55,12 @@ inline int tc_tile_n(int Nr, bool out_bound) {
   if (Nr <= 128) return 128;
   return 256;
 }
-// CTAs resident per SM for the two variants.
-inline int tc_ctas_per_sm(bool out_bound) { return out_bound ? 2 : 1; }
 
 // Whether a long sum split into nsplit accumulation chains runs as the
 // chained kernel (several chains per CTA, tiled A): every chain non-empty and
 // an N tile of at most 128 real columns.
 inline bool tc_chained(const TcOperands& op, int nsplit) {
-  if (op.out_bound || nsplit < 2 || tc_tile_n(2 * op.N, false) > 128) return false;
+  if (op.out_bound || nsplit < 2 || tc_tile_n(2 * op.N) > 128) return false;
   const int nkb = op.Kp / (128 / op.elem_bytes);
   const int per = (nkb + nsplit - 1) / nsplit;
   return (nkb + per - 1) / per == nsplit;
