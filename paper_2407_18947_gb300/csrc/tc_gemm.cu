@@ -624,27 +624,31 @@ k_tc_gemm_chains(const uint8_t* __restrict__ Atiled, const __grid_constant__ CUt
 //
 // As one CTA per 128 x 128 tile with a single load - split - MMA stage, each
 // tile pair took 44,000 cycles of mostly latency.  Complex64 times, before ->
-// now: 2432 x 92416 x 92 1.9 -> 0.69 ms (241 TFLOP/s, 722 with the three split
-// products, 65 % of the TF32 rate: bound by the MMAs and the reads of B from
-// L2); 3800 x 14440 x 48 0.18 -> 0.098 ms; accumulating 92416 x 2432 x 16 1.55
-// -> 0.85 ms (4.3 TB/s of read and written output).  64-column tiles run the
-// tensor pipe at half rate (0.163 instead of 0.097 ms at 3800 x 14440 x 48).
+// now: 92416 x 2432 x 92 1.9 -> 0.65 ms (254 TFLOP/s, 763 with the three split
+// products: bound by the MMAs, 0.63 ms without stores and loads); 14440 x 3800
+// x 48 0.18 -> 0.098 ms; accumulating 2432 x 92416 x 16 1.55 -> 0.62 ms (5.8
+// TB/s of read and written output, HBM).  64-column tiles run the tensor pipe
+// at half rate (0.163 instead of 0.098 ms at 14440 x 3800 x 48).
 //
 // Shared memory: the ring of B stages (128 rows of one K tile, hi and lo), two
-// raw A tiles on their way into tensor memory and, when accumulating, the
-// prefetched output tile.
+// raw A tiles on their way into tensor memory and, when accumulating, column
+// offsets.
 template <int NACC, bool ACC>
 struct TcShortSmem {
   static constexpr int BN = 128;
   static constexpr int kABytes = kBM * 128;
   static constexpr int kStage = 2 * BN * 128;
-  static constexpr int kOldBytes = ACC ? kBM * (BN / 2) * 8 : 0;  // prefetched output tile
-  static constexpr int kStages = (232448 - 1024 - 512 - 2 * kABytes - kOldBytes) / kStage;
+  static constexpr int kColBytes = ACC ? 16 * 4 * 16 * 8 : 0;  // 16 warps, four tiles of 16 columns
+  // accumulating: a short ring, because loads in flight hold lines of the L1,
+  // and the L1 is what the ring leaves of 256 KB (92416 x 2432 accumulated over
+  // 38 terms: 0.81 / 0.59 / 0.62 / 0.79 ms with 2 / 3 / 4 / 6 stages; one
+  // accumulator, 76 terms: 0.92 / 0.76 / 0.80 ms with 3 / 4 / 5)
+  static constexpr int kStages = ACC ? (NACC == 2 ? 3 : 4) : 6;
   static constexpr int kACol = NACC * BN;
   static constexpr int kMaxKb = (512 - kACol) / 64;
   static constexpr int kAOff = kStages * kStage;
-  static constexpr int kOldOff = kAOff + 2 * kABytes;
-  static constexpr int kBarOff = kOldOff + kOldBytes;
+  static constexpr int kColOff = kAOff + 2 * kABytes;
+  static constexpr int kBarOff = kColOff + kColBytes;
   static constexpr int kTotal = kBarOff + 512 + 1024;  // barriers + alignment slack
   static_assert(kStages >= 2 && kTotal <= 232448, "plan");
 };
@@ -783,8 +787,7 @@ k_tc_gemm_short(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const int e = warp - 3, chunk = e >> 2, q = warp & 3;
     const uint32_t lane_base = uint32_t(32 * q) << 16;
     const int row = 32 * q + lane;
-    float2* oldp = reinterpret_cast<float2*>(smem + L::kOldOff) + (threadIdx.x - 96);
-    const uint32_t old = smem_u32(oldp);
+    longlong2* cols = reinterpret_cast<longlong2*>(smem + L::kColOff) + e * 32;
     int j = 0, ia = 0, ui = 0;
     for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++ui) {
       const int m = u % mblocks * kBM + row;
@@ -825,13 +828,34 @@ k_tc_gemm_short(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       }
       const bool rin = m < M;
       float2* crow = C + (coff + (rin ? cM[m] : 0));
-      // ACC: the output tile's old values come by asynchronous copies into this
-      // thread's own places, one tile ahead of the MMAs
+      // ACC: the chunk's column offsets pass through shared memory (slot t % 4),
+      // read from the table three tiles ahead, and the output tile's old values
+      // are fetched one tile ahead of the MMAs
+      auto col = [&](int t) {
+        const int n = t * (BN / 2) + 16 * chunk + (lane & 15);
+        return t < t1 && n < N ? cN[n] : 0LL;
+      };
+      auto put = [&](int t, long long o) {
+        if (lane < 16) reinterpret_cast<long long*>(cols + (t & 3) * 8)[lane] = o;
+      };
+      long long next = 0;
+      if (ACC) {
+        __syncwarp();
+        put(t0, col(t0));
+        put(t0 + 1, col(t0 + 1));
+        next = col(t0 + 2);
+        __syncwarp();
+      }
+      float2 old[16];
       auto prefetch = [&](int t) {
-        const int n0 = t * (BN / 2) + 16 * chunk, nc = rin ? min(16, N - n0) : 0;
+        const int nc = rin ? min(16, N - (t * (BN / 2) + 16 * chunk)) : 0;
+        const longlong2* sl = cols + (t & 3) * 8;
 #pragma unroll
-        for (int k = 0; k < 16; ++k)
-          if (k < nc) cp_async8(old + k * 4096, crow + __ldg(cN + n0 + k), 8u);
+        for (int k = 0; k < 16; k += 2) {
+          const longlong2 o = sl[k >> 1];
+          old[k] = k < nc ? crow[o.x] : make_float2(0.f, 0.f);
+          old[k + 1] = k + 1 < nc ? crow[o.y] : make_float2(0.f, 0.f);
+        }
       };
       if (ACC) prefetch(t0);
       for (int t = t0; t < t1 && ok; ++t, ++j) {
@@ -845,28 +869,36 @@ k_tc_gemm_short(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&cfree[b]));
-        float2 v[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k)
-          v[k] = make_float2(alpha * __uint_as_float(r[2 * k]), alpha * __uint_as_float(r[2 * k + 1]));
+        const int nc = rin ? min(16, N - (t * (BN / 2) + 16 * chunk)) : 0;
         if (ACC) {
-          asm volatile("cp.async.wait_all;" ::: "memory");
+          float2 v[16];
 #pragma unroll
-          for (int k = 0; k < 16; ++k) {
-            const float2 w = oldp[k * 512];
-            v[k].x += w.x;
-            v[k].y += w.y;
-          }
+          for (int k = 0; k < 16; ++k)
+            v[k] = make_float2(alpha * __uint_as_float(r[2 * k]) + old[k].x,
+                               alpha * __uint_as_float(r[2 * k + 1]) + old[k].y);
           if (t + 1 < t1) prefetch(t + 1);
-        }
-        const int n0 = t * (BN / 2) + 16 * chunk, nc = rin ? min(16, N - n0) : 0;
+          const longlong2* sl = cols + (t & 3) * 8;
 #pragma unroll
-        for (int k = 0; k < 16; ++k)
-          if (k < nc) crow[__ldg(cN + n0 + k)] = v[k];
+          for (int k = 0; k < 16; k += 2) {
+            const longlong2 o = sl[k >> 1];
+            if (k < nc) crow[o.x] = v[k];
+            if (k + 1 < nc) crow[o.y] = v[k + 1];
+          }
+          put(t + 2, next);
+          next = col(t + 3);
+          __syncwarp();
+        } else {
+          float2* p[16];
+#pragma unroll
+          for (int k = 0; k < 16; ++k)
+            p[k] = crow + (k < nc ? __ldg(cN + t * (BN / 2) + 16 * chunk + k) : 0);
+#pragma unroll
+          for (int k = 0; k < 16; ++k)
+            if (k < nc)
+              *p[k] = make_float2(alpha * __uint_as_float(r[2 * k]), alpha * __uint_as_float(r[2 * k + 1]));
+        }
       }
     }
-    // no copy may be outstanding at exit
-    if (ACC) asm volatile("cp.async.wait_all;" ::: "memory");
   }
   if (!ok && err) atomicExch(err, 1);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
