@@ -89,6 +89,10 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
   return d;
 }
 
+// The low word of smem_desc; the high word is the same for every tile.
+__device__ __forceinline__ uint32_t smem_desc_lo(uint32_t addr) { return (addr >> 4) | (1u << 16); }
+constexpr uint32_t kDescHi = ((1024 >> 4) & 0x3FFF) | (1u << 14) | (2u << 29);
+
 // Instruction descriptor: D = F32, A/B format (2 = TF32 for kind::tf32,
 // 1 = BF16 for kind::f16), both K-major, N >> 3 at bit 17, M >> 4 at bit 24.
 template <bool BF16>
@@ -116,13 +120,13 @@ __device__ __forceinline__ void mma(uint32_t tmem, uint64_t a, uint64_t b, uint3
 }
 
 // D (+)= A B with A (128 rows = TMEM lanes, K = 8 TF32 columns) in tensor
-// memory and B from shared memory.
-__device__ __forceinline__ void mma_tf32_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t b,
+// memory and B from shared memory (low word of its descriptor).
+__device__ __forceinline__ void mma_tf32_ta(uint32_t tmem_d, uint32_t tmem_a, uint32_t b_lo,
                                             uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n" ::"r"(tmem_d),
-      "r"(tmem_a), "l"(b), "r"(idesc), "r"(accumulate)
+      "{\n .reg .pred p;\n .reg .b64 d;\n setp.ne.b32 p, %4, 0;\n mov.b64 d, {%2, %5};\n"
+      " tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], d, %3, p;\n}\n" ::"r"(tmem_d),
+      "r"(tmem_a), "r"(b_lo), "r"(idesc), "r"(accumulate), "n"(kDescHi)
       : "memory");
 }
 
@@ -511,16 +515,16 @@ k_tc_gemm_chains(const uint8_t* __restrict__ Atiled, const __grid_constant__ CUt
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t acc_t = tmem + uint32_t(b * L::kAccStride);
         const uint32_t sa = smem_u32(smem + st * L::kStageBytes);
-        const uint32_t sb = sa + L::kABytes;
+        const uint32_t sb = sa + L::kABytes, bd = smem_desc_lo(sb);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
           const uint32_t acc = (pos > 0 || kk > 0) ? 1u : 0u;
           if (SPLIT) {
             // A hi at columns kACol + 64 st, lo 32 columns further; 8 per K step
             const uint32_t ah = tmem + uint32_t(L::kACol + 64 * st + 8 * kk);
-            mma_tf32_ta(acc_t, ah, smem_desc(sb + kk * 32), idesc, acc);
-            mma_tf32_ta(acc_t, ah, smem_desc(sb + L::kBBytes + kk * 32), idesc, 1u);
-            mma_tf32_ta(acc_t, ah + 32, smem_desc(sb + kk * 32), idesc, 1u);
+            mma_tf32_ta(acc_t, ah, bd + 2 * kk, idesc, acc);
+            mma_tf32_ta(acc_t, ah, bd + (L::kBBytes >> 4) + 2 * kk, idesc, 1u);
+            mma_tf32_ta(acc_t, ah + 32, bd + 2 * kk, idesc, 1u);
           } else {
             mma<BF16>(acc_t, smem_desc(sa + kk * 32), smem_desc(sb + kk * 32), idesc, acc);
           }
@@ -744,13 +748,13 @@ k_tc_gemm_short(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             ok = ok && mbar_wait(smem_u32(&full[s]), ph, budget);
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t sb = smem_u32(smem + s * L::kStage);
+            const uint32_t bd = smem_desc_lo(smem_u32(smem + s * L::kStage));
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
               const uint32_t ah = tmem + uint32_t(L::kACol + 64 * kb + 8 * kk);
-              mma_tf32_ta(acc_t, ah, smem_desc(sb + kk * 32), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
-              mma_tf32_ta(acc_t, ah, smem_desc(sb + BN * 128 + kk * 32), idesc, 1u);
-              mma_tf32_ta(acc_t, ah + 32, smem_desc(sb + kk * 32), idesc, 1u);
+              mma_tf32_ta(acc_t, ah, bd + 2 * kk, idesc, kk > 0 ? 1u : (kb > 0 ? 1u : 0u));
+              mma_tf32_ta(acc_t, ah, bd + (BN * 128 >> 4) + 2 * kk, idesc, 1u);
+              mma_tf32_ta(acc_t, ah + 32, bd + 2 * kk, idesc, 1u);
             }
             mma_commit(smem_u32(&empty[s]));
             if (++s == S) { s = 0; ph ^= 1; }
@@ -1169,6 +1173,16 @@ struct TcDirectSmem {
 // TF32 hi and lo in tensor memory; warp 0 brings B by TMA, warp 1 issues the
 // MMAs (A from TMEM), warps 14-17 drain the accumulators to the chain
 // partials as in k_tc_gemm_chains.
+//
+// Bound by the one thread that waits for and issues the MMAs, about 1,300
+// cycles per K tile: without any loads it takes as long (0.142 of 0.150 ms),
+// and 20 columns take as long as 96.  So that thread counts instead of dividing,
+// reads the clock only when a wait does not succeed at once and gets the shared
+// memory descriptors by one addition, and the loaders read their K offsets a
+// tile ahead.  (10, 38), complex64, 3800 x 48 x 14440: 0.187 -> 0.156 ms; 14440 x
+// 10 x 3800: 0.177 -> 0.147 ms (3.1 TB/s of A).  Two groups of splitters, fewer or
+// more stages, and one barrier arrival per loader warp instead of per thread
+// changed nothing.
 template <int BN, bool AKC>
 __global__ void __launch_bounds__(576, 1)
 k_tc_gemm_direct(const float2* __restrict__ A, long long aoff, const long long* __restrict__ aM,
@@ -1249,25 +1263,30 @@ k_tc_gemm_direct(const float2* __restrict__ A, long long aoff, const long long* 
   } else if (warp == 1) {
     if (lane == 0) {
       constexpr uint32_t idesc = instr_desc<false>(kBM, BN);
+      int st = 0, ph = 0, j = 0, pos = 0;  // stage, its phase, chain, position in it
       for (int i = 0; i < nkb && ok; ++i) {
-        const int st = i % SB, j = i / per, pos = i - j * per, b = j & 1;
+        const int b = j & 1;
+        // the accumulator's previous chain (j - 2) must have been drained
         if (pos == 0 && j >= 2) ok = mbar_wait(smem_u32(&cfree[b]), ((j >> 1) - 1) & 1, budget);
-        if (ok) ok = mbar_wait(smem_u32(&conv[st]), (i / SB) & 1, budget);
-        if (ok) ok = mbar_wait(smem_u32(&bfull[st]), (i / SB) & 1, budget);
+        if (ok) ok = mbar_wait(smem_u32(&conv[st]), ph, budget);
+        if (ok) ok = mbar_wait(smem_u32(&bfull[st]), ph, budget);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t acc_t = tmem + uint32_t(b * L::kAccStride);
-        const uint32_t sb = smem_u32(smem + L::kBOff + st * L::kBStage);
+        const uint32_t bd = smem_desc_lo(smem_u32(smem + L::kBOff + st * L::kBStage));
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
           const uint32_t acc = (pos > 0 || kk > 0) ? 1u : 0u;
           const uint32_t ah = tmem + uint32_t(L::kACol + 64 * st + 8 * kk);
-          mma_tf32_ta(acc_t, ah, smem_desc(sb + kk * 32), idesc, acc);
-          mma_tf32_ta(acc_t, ah, smem_desc(sb + BN * 128 + kk * 32), idesc, 1u);
-          mma_tf32_ta(acc_t, ah + 32, smem_desc(sb + kk * 32), idesc, 1u);
+          mma_tf32_ta(acc_t, ah, bd + 2 * kk, idesc, acc);
+          mma_tf32_ta(acc_t, ah, bd + (BN * 128 >> 4) + 2 * kk, idesc, 1u);
+          mma_tf32_ta(acc_t, ah + 32, bd + 2 * kk, idesc, 1u);
         }
         mma_commit(smem_u32(&empty[st]));
-        if (pos == per - 1 || i == nkb - 1) mma_commit(smem_u32(&cfull[b]));
+        const bool last = ++pos == per;
+        if (last || i == nkb - 1) mma_commit(smem_u32(&cfull[b]));
+        if (last) { pos = 0; ++j; }
+        if (++st == SB) { st = 0; ph ^= 1; }
       }
       // every MMA issued has completed before tensor memory is freed (also
       // after giving up)
@@ -1290,6 +1309,14 @@ k_tc_gemm_direct(const float2* __restrict__ A, long long aoff, const long long* 
       rowok[u] = m < M;
       rowoff[u] = rowok[u] ? aoff + aM[m] : 0;
     }
+    // the K offsets of a tile are read one tile ahead
+    constexpr int NK = AKC ? 2 : 8;
+    long long ko[NK];
+#pragma unroll
+    for (int u = 0; u < NK; ++u) {
+      const int k = kb0 * 16 + (AKC ? 2 * (t & 7) + u : (t >> 7) + 2 * u);
+      ko[u] = k < K ? aK[k] : 0;
+    }
     for (int i = 0; i < nkb && ok; ++i) {
       const int st = i % SA;
       if (i >= SA) ok = mbar_wait(smem_u32(&aempty[st]), ((i / SA) - 1) & 1, budget);
@@ -1299,7 +1326,9 @@ k_tc_gemm_direct(const float2* __restrict__ A, long long aoff, const long long* 
       if (AKC) {
         const int j2 = t & 7, k = kbase + 2 * j2;
         const bool k0in = k < K, k1in = k + 1 < K;
-        const long long o0 = k0in ? aK[k] : 0, o1 = k1in ? aK[k + 1] : 0;
+        const long long o0 = ko[0], o1 = ko[1];
+        ko[0] = k + 16 < K ? aK[k + 16] : 0;
+        ko[1] = k + 17 < K ? aK[k + 17] : 0;
         const bool pair = k1in && o1 == o0 + 1;
 #pragma unroll
         for (int u = 0; u < NU; ++u) {
@@ -1322,10 +1351,11 @@ k_tc_gemm_direct(const float2* __restrict__ A, long long aoff, const long long* 
           const int j = (t >> 7) + 2 * u;
           const int k = kbase + j;
           const bool in = rowok[u] && k < K;
-          const float2* src = in ? A + rowoff[u] + aK[k] : A;
+          const float2* src = in ? A + rowoff[u] + ko[u] : A;
           // float 2j of row r: 16-byte chunk j / 2 at position (j / 2) ^ (r % 8)
           const uint32_t dst = sa + uint32_t(r * 128 + ((((j >> 1) ^ (r & 7)) << 4) | ((j & 1) << 3)));
           cp_async8(dst, src, in ? 8u : 0u);
+          ko[u] = k + 16 < K ? aK[k + 16] : 0;
         }
       }
       cp_async_arrive(smem_u32(&afull[st]));
