@@ -753,12 +753,20 @@ __global__ void __launch_bounds__(256) k_combine_brick(const BrickDesc<R> d) {
 // Several outputs of one pass over shared permuted sources (layout as
 // k_combine_brick): Y_o[blk][abc] = sum_u coef[o][u] X_u[blk][sigma_u(abc)],
 // each source element loaded once for all outputs.
+//
+// Complex128 is bound by the two FP64 FMAs per SM and cycle, not by memory: so
+// there an output skips the sources it has no coefficient for and begins with a
+// term of +-1 at no operation (t, 2t - t - t ...: 10 instead of 24 FMAs per
+// element, (10, 38) 2.78 -> 1.86 ms).  Complex64 is bound by memory (0.50 ms) and
+// keeps the straight sums.
+enum SumTerm : int { kSumSkip = 0, kSumPlus, kSumMinus, kSumScale, kSumAdd };
 constexpr int kMultiOut = 3;
 template <typename R>
 struct BrickMultiDesc {
   const Cx<R>* src[6];
   int lv[6];
   R coef[kMultiOut][6];
+  int kind[kMultiOut][6];  // SumTerm, from the last source to the first (complex128)
   Cx<R>* y[kMultiOut];
   int v;
 };
@@ -790,9 +798,26 @@ __global__ void __launch_bounds__(256) k_combine_brick_multi(const BrickMultiDes
     for (int o = 0; o < NO; ++o) {
       R re = R(0), im = R(0);
 #pragma unroll
-      for (int u = 0; u < NU; ++u) {
-        re += d.coef[o][u] * x[u].x;
-        im += d.coef[o][u] * x[u].y;
+      for (int w = 0; w < NU; ++w) {
+        if (sizeof(R) == 4) {
+          re += d.coef[o][w] * x[w].x;
+          im += d.coef[o][w] * x[w].y;
+          continue;
+        }
+        const int u = NU - 1 - w, kind = d.kind[o][u];
+        if (kind == kSumAdd) {
+          re += d.coef[o][u] * x[u].x;
+          im += d.coef[o][u] * x[u].y;
+        } else if (kind == kSumPlus) {
+          re = x[u].x;
+          im = x[u].y;
+        } else if (kind == kSumMinus) {
+          re = -x[u].x;
+          im = -x[u].y;
+        } else if (kind == kSumScale) {
+          re = d.coef[o][u] * x[u].x;
+          im = d.coef[o][u] * x[u].y;
+        }
       }
       d.y[o][out] = cmake<R>(re, im);
     }
@@ -803,12 +828,14 @@ __global__ void __launch_bounds__(256) k_combine_brick_multi(const BrickMultiDes
 // dense (o,o,o,v,v,v): the two outer products of the adjoints of X1 and of
 // the first X2 term (Eqs. A21-A22) in one pass (a term with a zero
 // coefficient is not read).  One block row per (i,j,k), consecutive threads
-// on consecutive abc.
+// on consecutive abc.  Complex128 is bound by its FP64 operations: the factors
+// are scaled only where a coefficient is not 1 (unit1, unit2), and coefficients
+// are tested on the host ((10, 38): 1.47 -> 1.21 ms).
 template <typename R>
 __global__ void __launch_bounds__(256)
 k_outer_pair(Cx<R>* __restrict__ Y, const Cx<R>* __restrict__ x1, const Cx<R>* __restrict__ y1,
-             const Cx<R>* __restrict__ x2, const Cx<R>* __restrict__ y2, R a1, R a2, int o, int v,
-             int accumulate, const FastDiv fv2, const FastDiv fv) {
+             const Cx<R>* __restrict__ x2, const Cx<R>* __restrict__ y2, R a1, R a2, int unit1, int unit2,
+             int o, int v, int accumulate, const FastDiv fv2, const FastDiv fv) {
   const int ijk = blockIdx.y;
   const int i = ijk / (o * o), j = (ijk / o) % o, k = ijk % o;
   const unsigned v2 = unsigned(v) * v, v3 = v2 * v;
@@ -820,15 +847,19 @@ k_outer_pair(Cx<R>* __restrict__ Y, const Cx<R>* __restrict__ x1, const Cx<R>* _
   for (unsigned abc = blockIdx.x * blockDim.x + threadIdx.x; abc < v3; abc += gridDim.x * blockDim.x) {
     const unsigned a = fv2.div(abc), bc = abc - a * v2, b = fv.div(bc), c = bc - b * v;
     R re = R(0), im = R(0);
-    if (a1 != R(0)) {
-      const Cx<R> p = x1i[a], q = y1jk[bc];
-      re += a1 * (p.x * q.x - p.y * q.y);
-      im += a1 * (p.x * q.y + p.y * q.x);
+    if (x1) {
+      Cx<R> p = x1i[a];
+      const Cx<R> q = y1jk[bc];
+      if (!unit1) p = cmake<R>(a1 * p.x, a1 * p.y);
+      re = p.x * q.x - p.y * q.y;
+      im = p.x * q.y + p.y * q.x;
     }
-    if (a2 != R(0)) {
-      const Cx<R> p = x2ij[a * v + b], q = y2k[c];
-      re += a2 * (p.x * q.x - p.y * q.y);
-      im += a2 * (p.x * q.y + p.y * q.x);
+    if (x2) {
+      Cx<R> p = x2ij[a * v + b];
+      const Cx<R> q = y2k[c];
+      if (!unit2) p = cmake<R>(a2 * p.x, a2 * p.y);
+      re = fma(-p.y, q.y, fma(p.x, q.x, re));
+      im = fma(p.y, q.x, fma(p.x, q.y, im));
     }
     if (accumulate) {
       const Cx<R> y = yb[abc];
@@ -2069,6 +2100,16 @@ void Engine<R>::combine_multi(const std::vector<std::vector<std::pair<double, Vi
     const dim3 grid(unsigned((v + 3) / 4) * unsigned((v + 7) / 8), unsigned(nblk));
     const int pk = pbegin();
     const int nu = int(uniq.size()), no = int(ys.size());
+    for (int o = 0; o < no; ++o) {
+      bool begun = false;
+      for (int u = nu - 1; u >= 0; --u) {
+        const R c = d.coef[o][u];
+        d.kind[o][u] = c == R(0) ? kSumSkip
+                                 : (begun ? kSumAdd
+                                          : (c == R(1) ? kSumPlus : (c == R(-1) ? kSumMinus : kSumScale)));
+        begun = begun || c != R(0);
+      }
+    }
 #define RTCC3_BM(NUV, NOV)                                                                   \
   if (layout == 1) k_combine_brick_multi<R, NUV, NOV, 1><<<grid, 256, 0, stream_>>>(d);      \
   else k_combine_brick_multi<R, NUV, NOV, 0><<<grid, 256, 0, stream_>>>(d)
@@ -2138,7 +2179,7 @@ void Engine<R>::exec_outer_pair(double a1, const View& x1g, const View& y1, doub
   k_outer_pair<R><<<grid, 256, 0, stream_>>>(
       nodes_[dstg.node].grad, a1 != 0.0 ? nodes_[x1g.node].grad + x1g.off : nullptr,
       nodes_[y1.node].data + y1.off, a2 != 0.0 ? nodes_[x2g.node].grad + x2g.off : nullptr,
-      nodes_[y2.node].data + y2.off, R(a1), R(a2), o, v, acc ? 1 : 0, FastDiv(v2),
+      nodes_[y2.node].data + y2.off, R(a1), R(a2), a1 == 1.0, a2 == 1.0, o, v, acc ? 1 : 0, FastDiv(v2),
       FastDiv(unsigned(v)));
   ++launches_;
   RTCC3_CUDA(cudaGetLastError());
