@@ -225,6 +225,12 @@ class Engine {
   // its term unread).
   void exec_outer_pair(double a1, const View& x1g, const View& y1, double a2, const View& x2g,
                        const View& y2, const View& dstg);
+  // Y (a dense slab of the t3 cotangent, first occupied index i0) = the outer
+  // products of grad(X), grad(S) with L, F in the three arrangements (see
+  // k_slab_outers); St holds grad(S) with its last two indices exchanged.
+  // Cotangents never written count as zero.
+  void exec_slab_outers(const View& Xg, const View& Sg, const View& St, const View& L, const View& F,
+                        int i0, const View& Y);
   void exec_sym3_div(const View& X, bool xg, const EpsSpec& es, const View& Y) {
     run_sym6_div(1.0, X, xg, es, Y, false, true, 3);
   }

@@ -202,18 +202,19 @@ void blocked_triples(Engine<R>& E, int o, int v, int chunk, const TriplesOperand
       Dv = E.node({v, v});
       Do = E.node({o, o});
     }
-    // Q[p,q,r,x,y,z] (the t3 cotangent) as nine products of small tensors;
-    // placeholders p q r x y z are mapped to the output letters of one of
-    // the three arrangements, d and l are sums
-    struct QT { const char* a; int ga; const char* b; double alpha; };
-    // ga: 0 grad X1, 1 grad S3; b operand: 0 Lp, 1 Fp, 2 Gb2, 3 Gb, 4 Gc
-    static const char* kQa[9] = {"px", "pqxy", "pz", "pqzy", "pqdy", "pqdz", "lqzy", "lqzx", "lqxy"};
-    static const int kQga[9] = {0, 1, 0, 1, 1, 1, 1, 1, 1};
-    static const char* kQb[9] = {"qryz", "rz", "qryx", "rx", "dxrz", "dxry", "rlpx", "rlpy", "rlpz"};
-    static const int kQbw[9] = {0, 1, 0, 1, 2, 3, 4, 4, 4};
-    static const double kQal[9] = {1.0, 1.0, -1.0, -1.0, 1.0, -1.0, -2.0, 1.0, 1.0};
+    // Q[p,q,r,x,y,z] (the t3 cotangent) as four outer products (exec_slab_outers)
+    // and five products of small tensors with grad S3; placeholders p q r x y z
+    // are mapped to the output letters of one of the three arrangements, d and l
+    // are sums
+    // b operand: 0 Gb2, 1 Gb, 2 Gc
+    static const char* kQa[5] = {"pqdy", "pqdz", "lqzy", "lqzx", "lqxy"};
+    static const char* kQb[5] = {"dxrz", "dxry", "rlpx", "rlpy", "rlpz"};
+    static const int kQbw[5] = {0, 1, 2, 2, 2};
+    static const double kQal[5] = {1.0, -1.0, -2.0, 1.0, 1.0};
     static const char* kPos[3] = {"ijkabc", "jikbac", "kjicba"};  // p q r x y z
-    const View bops[5] = {in.Lp, in.Fp, GB2, in.Gb, in.Gc};
+    const View bops[3] = {GB2, in.Gb, in.Gc};
+    const View St = E.v(E.node({o, o, v, v}, false, false));
+    if (E.grad_ready(S3o)) E.exec_copy(E.ev("ijba->ijab", S3v), true, St);
     auto map = [](const char* t, const char* pos) {
       std::string r(t);
       for (char& ch : r) {
@@ -244,13 +245,12 @@ void blocked_triples(Engine<R>& E, int o, int v, int chunk, const TriplesOperand
         prod("imkcba,jmab->kjic", -1.0, {U, false, true}, {S3v, true, false}, {in.Gc, true, false}, i0, I, true);
       }
       // R = sum over the three arrangements of Q; S = R + R(ikjacb) = P(Q)
-      bool first = true;
+      E.exec_slab_outers(X1v, S3v, St, in.Lp, in.Fp, i0, U);
       for (int ps = 0; ps < 3; ++ps)
-        for (int t = 0; t < 9; ++t) {
+        for (int t = 0; t < 5; ++t) {
           const std::string spec = map(kQa[t], kPos[ps]) + "," + map(kQb[t], kPos[ps]) + "->ijkabc";
-          prod(spec, kQal[t], {kQga[t] ? S3v : X1v, true, false}, {bops[kQbw[t]], false, false}, {U, false, true}, i0,
-               I, !first);
-          first = false;
+          prod(spec, kQal[t], {S3v, true, false}, {bops[kQbw[t]], false, false}, {U, false, true}, i0, I,
+               true);
         }
       E.exec_slab_sym(1.0, {U}, i0, es, W);  // W = P(Q) / D = -grad Z
       if (gfield) {
