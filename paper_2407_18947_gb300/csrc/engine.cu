@@ -2085,8 +2085,8 @@ void Engine<R>::combine(std::initializer_list<std::pair<double, View>> srcs, con
 }
 
 template <typename R>
-void Engine<R>::combine_multi(const std::vector<std::vector<std::pair<double, View>>>& srcs,
-                              const std::vector<View>& ys) {
+void Engine<R>::exec_combine_multi(const std::vector<std::vector<std::pair<double, View>>>& srcs,
+                                   const std::vector<View>& ys) {
   RTCC3_CHECK(srcs.size() == ys.size() && !ys.empty(), kErrArg, "combine_multi: one source list per output");
   // the fused pass: overwriting outputs of one dense (..., v, v, v) shape,
   // at most six distinct sources (views of data, not cotangents) that share
@@ -2201,6 +2201,12 @@ void Engine<R>::combine_multi(const std::vector<std::vector<std::pair<double, Vi
                                         " nout=" + std::to_string(no)
                                   : std::string());
   }
+}
+
+template <typename R>
+void Engine<R>::combine_multi(const std::vector<std::vector<std::pair<double, View>>>& srcs,
+                              const std::vector<View>& ys) {
+  exec_combine_multi(srcs, ys);
   // the tape holds one combine per output, as if each had run alone
   for (size_t o = 0; o < ys.size(); ++o) {
     bool g = false;

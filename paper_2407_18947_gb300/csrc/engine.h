@@ -124,6 +124,9 @@ class Engine {
   // else one combine after another; the tape records one combine per output.
   void combine_multi(const std::vector<std::vector<std::pair<double, View>>>& srcs,
                      const std::vector<View>& ys);
+  // The same pass, untaped.
+  void exec_combine_multi(const std::vector<std::vector<std::pair<double, View>>>& srcs,
+                          const std::vector<View>& ys);
   // Y (+)= alpha P_ijk^abc X for 6-index tensors (o,o,o,v,v,v); self-adjoint.
   void sym6(double alpha, const View& X, const View& Y, bool overwrite);
   void mulc(const View& X, const View& Cst, const View& Y);

@@ -123,7 +123,8 @@ void blocked_triples(Engine<R>& E, int o, int v, int chunk, const TriplesOperand
                  E.needs_grad(in.Gb.node) || E.needs_grad(in.Gc.node) ||
                  (fa.on && E.needs_grad(fa.wt));
   // slab buffers: nb0 holds t3; nb1..nb3 hold the three Z slabs while W is
-  // built, then serve as scratch (nb1) and P(Q)/D (nb2) in the reverse pass
+  // built, then the combinations of t3; in the reverse pass nb1 and nb2 then
+  // serve as scratch and P(Q)/D
   const int nb0 = E.node({I0, o, o, v, v, v}, false, false);
   const int nb1 = E.node({I0, o, o, v, v, v}, false, false);
   const int nb2 = E.node({I0, o, o, v, v, v}, false, false);
@@ -172,27 +173,32 @@ void blocked_triples(Engine<R>& E, int o, int v, int chunk, const TriplesOperand
     }
     E.exec_slab_sym(-1.0, {Z1, Z2, Z3}, i0, es, T);
   };
+  // t - t(cba), 2 t - t(acb) - t(cba) and 2 t - t(bac) - t(cba) into the three Z
+  // slabs, free once t3 is built: one pass over t3 (as three, each re-read it:
+  // 4.0 ms a complex64 slab of two of (20, 76), now 2.4)
+  auto combos = [&E](const View& T, const View& U, const View& Ub, const View& Uc) {
+    E.exec_combine_multi({{{1.0, T}, {-1.0, E.ev("ijkcba->ijkabc", T)}},
+                          {{2.0, T}, {-1.0, E.ev("ijkxzy->ijkxyz", T)}, {-1.0, E.ev("ijkzyx->ijkxyz", T)}},
+                          {{2.0, T}, {-1.0, E.ev("ijkyxz->ijkxyz", T)}, {-1.0, E.ev("ijkzyx->ijkxyz", T)}}},
+                         {U, Ub, Uc});
+  };
   const View X1v = E.v(X1o), S3v = E.v(S3o);
   for (int i0 = 0; i0 < o; i0 += I0) {
     const int I = std::min(I0, o - i0);
-    const View T = slab(nb0, I), U = slab(nb1, I);
-    build_t3(T, U, slab(nb2, I), slab(nb3, I), i0, I);
-    E.exec_combine({{1.0, T}, {-1.0, E.ev("ijkcba->ijkabc", T)}}, U, true);
+    const View T = slab(nb0, I), U = slab(nb1, I), Ub = slab(nb2, I), Uc = slab(nb3, I);
+    build_t3(T, U, Ub, Uc, i0, I);
+    combos(T, U, Ub, Uc);
     prod("ijkabc,jkbc->ia", 1.0, {U, false, true}, {in.Lp, false, false}, {X1v, false, false}, i0, I, true);
     prod("ijkabc,kc->ijab", 1.0, {U, false, true}, {in.Fp, false, false}, {S3v, false, false}, i0, I, true);
-    E.exec_combine({{2.0, T}, {-1.0, E.ev("ijkxzy->ijkxyz", T)}, {-1.0, E.ev("ijkzyx->ijkxyz", T)}},
-                   U, true);
-    prod("ijkcbe,acke->ijab", 1.0, {U, false, true}, {in.Gb, false, false}, {S3v, false, false}, i0, I, true);
-    E.exec_combine({{2.0, T}, {-1.0, E.ev("ijkyxz->ijkxyz", T)}, {-1.0, E.ev("ijkzyx->ijkxyz", T)}},
-                   U, true);
+    prod("ijkcbe,acke->ijab", 1.0, {Ub, false, true}, {in.Gb, false, false}, {S3v, false, false}, i0, I, true);
     // the slab index is Uc's first occupied index (m), a sum index here
-    prod("imkcba,kjic->jmab", -1.0, {U, false, true}, {in.Gc, false, false}, {S3v, false, false}, i0, I, true);
+    prod("imkcba,kjic->jmab", -1.0, {Uc, false, true}, {in.Gc, false, false}, {S3v, false, false}, i0, I, true);
   }
   if (!g) return;
   const int Gb2 = E.node({v, v, o, v}, false, false);
   E.exec_combine({{2.0, in.Gb}, {-1.0, E.ev("dzrx->dxrz", in.Gb)}}, E.v(Gb2), true);
   const View GB2 = E.v(Gb2);
-  E.custom([&E, o, v, I0, in, es, fa, nb0, nb1, nb2, nb3, X1o, S3o, GB2, prod, build_t3, slab]() {
+  E.custom([&E, o, v, I0, in, es, fa, nb0, nb1, nb2, nb3, X1o, S3o, GB2, prod, build_t3, combos, slab]() {
     const View X1v = E.v(X1o), S3v = E.v(S3o);
     const bool gl = E.needs_grad(in.Lp.node), gf = E.needs_grad(in.Fp.node),
                gb = E.needs_grad(in.Gb.node), gc = E.needs_grad(in.Gc.node);
@@ -226,24 +232,14 @@ void blocked_triples(Engine<R>& E, int o, int v, int chunk, const TriplesOperand
     };
     for (int i0 = 0; i0 < o; i0 += I0) {
       const int I = std::min(I0, o - i0);
-      const View T = slab(nb0, I), U = slab(nb1, I), W = slab(nb2, I);
-      build_t3(T, U, W, slab(nb3, I), i0, I);
-      // cotangents of the X-side operands
-      if (gl || gf) {
-        E.exec_combine({{1.0, T}, {-1.0, E.ev("ijkcba->ijkabc", T)}}, U, true);
-        if (gl) prod("ijkabc,ia->jkbc", 1.0, {U, false, true}, {X1v, true, false}, {in.Lp, true, false}, i0, I, true);
-        if (gf) prod("ijkabc,ijab->kc", 1.0, {U, false, true}, {S3v, true, false}, {in.Fp, true, false}, i0, I, true);
-      }
-      if (gb) {
-        E.exec_combine({{2.0, T}, {-1.0, E.ev("ijkxzy->ijkxyz", T)},
-                        {-1.0, E.ev("ijkzyx->ijkxyz", T)}}, U, true);
-        prod("ijkcbe,ijab->acke", 1.0, {U, false, true}, {S3v, true, false}, {in.Gb, true, false}, i0, I, true);
-      }
-      if (gc) {
-        E.exec_combine({{2.0, T}, {-1.0, E.ev("ijkyxz->ijkxyz", T)},
-                        {-1.0, E.ev("ijkzyx->ijkxyz", T)}}, U, true);
-        prod("imkcba,jmab->kjic", -1.0, {U, false, true}, {S3v, true, false}, {in.Gc, true, false}, i0, I, true);
-      }
+      const View T = slab(nb0, I), U = slab(nb1, I), W = slab(nb2, I), Uc = slab(nb3, I);
+      build_t3(T, U, W, Uc, i0, I);
+      // cotangents of the X-side operands (the combinations pass through U, W, Uc)
+      if (gl || gf || gb || gc) combos(T, U, W, Uc);
+      if (gl) prod("ijkabc,ia->jkbc", 1.0, {U, false, true}, {X1v, true, false}, {in.Lp, true, false}, i0, I, true);
+      if (gf) prod("ijkabc,ijab->kc", 1.0, {U, false, true}, {S3v, true, false}, {in.Fp, true, false}, i0, I, true);
+      if (gb) prod("ijkcbe,ijab->acke", 1.0, {W, false, true}, {S3v, true, false}, {in.Gb, true, false}, i0, I, true);
+      if (gc) prod("imkcba,jmab->kjic", -1.0, {Uc, false, true}, {S3v, true, false}, {in.Gc, true, false}, i0, I, true);
       // R = sum over the three arrangements of Q; S = R + R(ikjacb) = P(Q)
       E.exec_slab_outers(X1v, S3v, St, in.Lp, in.Fp, i0, U);
       for (int ps = 0; ps < 3; ++ps)
