@@ -884,8 +884,8 @@ template <typename R>
 __global__ void __launch_bounds__(256)
 k_slab_outers(Cx<R>* __restrict__ Y, const Cx<R>* __restrict__ X, const Cx<R>* __restrict__ S,
               const Cx<R>* __restrict__ St, const Cx<R>* __restrict__ L, const Cx<R>* __restrict__ F,
-              int fs, int o, int v, int i0, int na, const FastDiv fv) {
-  const int ijk = blockIdx.y, i = i0 + ijk / (o * o), j = (ijk / o) % o, k = ijk % o;
+              int fs, int o, int v, int i0, int na, unsigned first, const FastDiv fv) {
+  const int ijk = int(first + blockIdx.y), i = i0 + ijk / (o * o), j = (ijk / o) % o, k = ijk % o;
   const unsigned v2 = unsigned(v) * v;
   const unsigned bc = blockIdx.x * 256 + threadIdx.x;
   if (bc >= v2) return;
@@ -2279,18 +2279,20 @@ void Engine<R>::exec_slab_outers(const View& Xg, const View& Sg, const View& St,
                   F.shape[1] == v && F.stride[1] == 1 && i0 >= 0 && i0 + I <= o,
               kErrArg, "slab outers need dense operands");
   for (const View* w : {&Xg, &Sg, &St, &L, &F, &Y}) check_view(*w, 0, "slab_outers");
-  RTCC3_CHECK(size_t(I) * o * o < 65536u, kErrArg, "slab outers: too many occupied blocks");
   const bool x = nodes_[Xg.node].grad_ready, sg = nodes_[Sg.node].grad_ready;
   const unsigned v2 = unsigned(v) * unsigned(v), nt = (v2 + 255) / 256;
   const int na = std::min(v, 20);  // a per thread: the (b, c) part is read once in 20
   const int pk = pbegin();
-  k_slab_outers<R><<<dim3(nt, unsigned(I) * o * o, unsigned((v + na - 1) / na)), 256, 0, stream_>>>(
-      nodes_[Y.node].data + Y.off, x ? nodes_[Xg.node].grad + Xg.off : nullptr,
-      sg ? nodes_[Sg.node].grad + Sg.off : nullptr, sg ? nodes_[St.node].data + St.off : nullptr,
-      nodes_[L.node].data + L.off, nodes_[F.node].data + F.off, int(F.stride[0]), o, v, i0, na,
-      FastDiv(unsigned(v)));
-  ++launches_;
-  RTCC3_CUDA(cudaGetLastError());
+  const unsigned blocks = unsigned(I) * o * o;
+  for (unsigned first = 0; first < blocks; first += 65535u) {
+    k_slab_outers<R><<<dim3(nt, std::min(blocks - first, 65535u), unsigned((v + na - 1) / na)), 256, 0, stream_>>>(
+        nodes_[Y.node].data + Y.off, x ? nodes_[Xg.node].grad + Xg.off : nullptr,
+        sg ? nodes_[Sg.node].grad + Sg.off : nullptr, sg ? nodes_[St.node].data + St.off : nullptr,
+        nodes_[L.node].data + L.off, nodes_[F.node].data + F.off, int(F.stride[0]), o, v, i0, na, first,
+        FastDiv(unsigned(v)));
+    ++launches_;
+    RTCC3_CUDA(cudaGetLastError());
+  }
   const double n = double(Y.numel());
   pend(pk, "slab_outers", 90.0 * n, n * sizeof(C));
 }
