@@ -122,6 +122,7 @@ KERNEL_FAMILIES = {
     # the o^3 v^3 permuted sums in the brick thread layouts (k_combine_brick
     # and its several-output form k_combine_brick_multi)
     "k_combine_brick": (("combine_brick",), "hbm"),
+    # (the short TF32 sums run as k_tc_gemm_short)
     "k_tc_gemm": (("contract_tc_tf32", "contract_tc_bf16"), "tensor"),
     # long sums reading the o^3 v^3 operand from its source (tcgen05, TF32
     # split): N = 10 or 38 complex columns, ~N flop per byte, HBM-bound
@@ -132,6 +133,10 @@ KERNEL_FAMILIES = {
     "k_contract": (("contract_simt_c64", "contract_simt_c128"), "alu"),
     "k_sym6_orbit": (("sym6_div",), "hbm"),
     "k_sym3_div": (("sym3_div",), "hbm"),
+    # blocked triples: slab sums with their denominators, outer products of the
+    # t3 cotangent
+    "k_slab_sym": (("slab_sym",), "hbm"),
+    "k_slab_outers": (("slab_outers",), "alu"),
     # FP64 products as sliced FP16 tensor-core products
     "k_oz_gemm": (("contract_sliced_c128",), "tensor"),
     # small products, a few terms per lane
@@ -151,9 +156,6 @@ KERNEL_FAMILIES = {
 MEASURED_TRAFFIC = {
     ("k_combine_nd", "tf32", 2): 3.61e6,
     ("k_combine_brick", "tf32", 2): 1755.6e6,
-    ("k_tc_gemm", "tf32", 2): 517.74e6,
-    ("k_tc_gemm_direct", "tf32", 2): 485.34e6,
-    ("k_outer_pair", "tf32", 2): 377.12e6,
     ("k_gemv", "tf32", 2): 221.78e6,
     ("k_pack", "tf32", 2): 2.01e6,
 }
