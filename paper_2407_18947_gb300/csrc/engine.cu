@@ -1363,14 +1363,19 @@ ContractPlan& Engine<R>::plan(const std::string& spec, const View& A, const View
     for (auto& l : g) n *= l.ext;
     const size_t base = out.size();
     out.resize(base + size_t(n));
+    // counting up (a division per index and entry was a good part of the time
+    // in which a first evaluation builds its plans)
+    std::vector<long long> idx(g.size(), 0);
+    long long off = 0;
     for (long long t = 0; t < n; ++t) {
-      long long rem = t, off = 0;
-      for (int k = int(g.size()) - 1; k >= 0; --k) {
-        const long long i = rem % g[k].ext;
-        rem /= g[k].ext;
-        off += i * (which == 0 ? g[k].sa : (which == 1 ? g[k].sb : g[k].sc));
-      }
       out[base + size_t(t)] = off;
+      for (int k = int(g.size()) - 1; k >= 0; --k) {
+        const long long st = which == 0 ? g[k].sa : (which == 1 ? g[k].sb : g[k].sc);
+        off += st;
+        if (++idx[k] < g[k].ext) break;
+        off -= g[k].ext * st;
+        idx[k] = 0;
+      }
     }
     return base;
   };
