@@ -214,34 +214,42 @@ k_eig_refine(EigJob ja, EigJob jb) {
     T mx = T(0);
     for (int t = warp; t < rows; t += kRefineThreads / 32) {
       const int i = rank + kCl * t;
-      const V li = lam_at(i);
       V q = X::mk(T(0), T(0));
       for (int j = lane; j < n; j += 32) {
         V e;
         if (j == i) {
           e = r_at(i, i);
         } else {
-          const V lj = lam_at(j);
-          const V b = X::add(s_at(i, j), X::mul(r_at(i, j), lj));
-          const V c = X::add(s_at(j, i), X::mul(r_at(j, i), li));
+          // Rows i and j of a pair have to take opposite roots, or both columns
+          // become the same vector: both work out the same b, c, s of (lo, hi)
+          // bit for bit and row hi changes the signs.
+          const int lo = min(i, j), hi = max(i, j);
+          const V ll = lam_at(lo), lh = lam_at(hi);
+          const V b = X::add(s_at(lo, hi), X::mul(r_at(lo, hi), lh));
+          const V c = X::add(s_at(hi, lo), X::mul(r_at(hi, lo), ll));
           const T ab = X::abs(b), ac = X::abs(c);
           if (ab <= floor_ && ac <= floor_) {
             e = X::mk(T(0), T(0));
           } else {
-            const V dl = X::scale(X::sub(li, lj), T(0.5));
+            const V dl = X::scale(X::sub(ll, lh), T(0.5));
             const V bc = X::mul(b, c);
             V s = dl;
             const T d2 = dl.x * dl.x + dl.y * dl.y;
             if (ab * ac > T(1e-8) * d2) {
               s = X::sqrt_(X::add(X::mul(dl, dl), bc));
-              if (dl.x * s.x + dl.y * s.y < T(0) || (d2 == T(0) && i > j)) s = X::scale(s, T(-1));
+              if (dl.x * s.x + dl.y * s.y < T(0)) s = X::scale(s, T(-1));
             }
             const V den = X::add(dl, s);
-            e = X::scale(X::div(b, den), T(-1));
+            e = j > i ? X::scale(X::div(b, den), T(-1)) : X::div(c, den);
             q = X::sub(q, X::mul(X::div(b, den), X::div(c, den)));
             const T ae = X::abs(e);
             mx = ae > mx || !(ae == ae) ? ae : mx;
           }
+        }
+        if (it > 0) {
+          // Y has to be the inverse of X too
+          const T ar = X::abs(r_at(i, j));
+          mx = ar > mx || !(ar == ar) ? ar : mx;
         }
         W.E[size_t(i) * n + j] = e;
       }
