@@ -175,6 +175,9 @@ k_eig_refine(EigJob ja, EigJob jb) {
 #pragma unroll
   for (int w = 1; w < kRefineThreads / 32; ++w) mag = wmax[w] > mag || !(wmax[w] == wmax[w]) ? wmax[w] : mag;
   __syncthreads();
+  // not a number, or one without a rounding floor: k_eig_warp says so (mag is
+  // the same in the whole cluster)
+  if (!isfinite(mag)) return;
   const T floor_ = eps * mag;
   const int max_it = J.max_sweeps > 0 ? min(J.max_sweeps, kRefineMax) : kRefineMax;
   int cur = 0;

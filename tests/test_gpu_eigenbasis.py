@@ -86,3 +86,28 @@ def test_real_pair_with_couplings_of_opposite_sign(precision, tol, o, v, pair, s
     for k in ("r_t1", "r_t2", "r_l1", "r_l2"):
         want = getattr(ref, k).numpy()
         assert np.abs(r[k] - want).max() <= tol * np.abs(want).max(), k
+
+
+@pytest.mark.parametrize("precision,big", [(0, 1e308), (1, 1e38)])
+@pytest.mark.parametrize("o,v", [(1, 1), (1, 2), (2, 1)])
+def test_overflowing_coupling_is_reported(precision, big, o, v):
+    """A dressed matrix with an infinite element is refused, also where its
+    diagonal is finite ((1, 2) and (2, 1): w~_01 = -t_0 w_1 alone overflows)."""
+    from paper_2407_18947_gb300._lib import ERR_NONFINITE, RTCC3Error
+    from paper_2407_18947_gb300.api import RTCC3
+    s = make_system(o, v, seed=530)
+    amps = [np.zeros_like(x) for x in random_amplitudes(o, v, seed=531)]
+    s.dipole[:] = 0.0
+    s.eps[:o] -= 1000.0                             # (a field of 20 is not too strong)
+    s.eps[o:] += 1000.0
+    amps[0][0, 0] = big
+    i, a = o - 1, o + v - 1                         # the last occupied and virtual
+    s.dipole[2, i, a] = s.dipole[2, a, i] = 1000.0
+    eng = RTCC3(o, v, precision=precision)
+    eng.set_hamiltonian(s.eps, s.Lfac, s.dipole)
+    eng.set_field(0, 1, 0.02, direction=(0.0, 0.0, 1.0))
+    eng.set_amplitudes(0, *amps)
+    with pytest.raises(RTCC3Error) as ei:
+        eng.compute_residuals(0, 0.0)
+    assert ei.value.code == ERR_NONFINITE and "dressed field matrix" in str(ei.value)
+    eng.close()
