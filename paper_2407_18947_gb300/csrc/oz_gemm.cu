@@ -255,6 +255,7 @@ struct OzArgs {
   const long long *aM, *aK, *bN, *bK, *cM, *cN;
   double2* C;      // already moved by its offset; the partials when nsplit > 1
   int M, N, K;
+  unsigned zrow, zspc;  // row blocks and segments a step of blockIdx.z stands for (one is 0)
   int seg, nseg, spc;
   int ash;         // alpha = (neg ? -1 : 1) 2^ash alpha_rest, neg = all ones or 0
   uint32_t neg;
@@ -280,8 +281,10 @@ __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs 
   long long* sCM = sK + 4 * kSegMax;
   long long* sCN = sCM + kRows;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
-  const int m0 = blockIdx.y * kRows, n0 = blockIdx.x * NB;
-  const int s0 = blockIdx.z * P.spc, s1 = min(P.nseg, s0 + P.spc);
+  const unsigned rb = blockIdx.y + blockIdx.z * P.zrow;
+  if ((long long)rb * kRows >= P.M) return;
+  const int m0 = int(rb) * kRows, n0 = blockIdx.x * NB;
+  const int s0 = blockIdx.z * P.zspc, s1 = min(P.nseg, s0 + P.spc);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < 2; ++s) {
@@ -731,10 +734,15 @@ int oz_gemm(const OzPlan& p, const OzOperand& A, const OzOperand& B, int M, int 
       a.alpha_rest = alpha;
     }
   }
-  const long long gx = (2LL * N + p.nt - 1) / p.nt, gy = (M + kRows - 1) / kRows;
-  const long long gz = (p.nseg + p.spc - 1) / p.spc;
-  RTCC3_CHECK(gy < 65536 && gz < 65536, kErrArg, "sliced product: grid too large");
-  dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)gz);
+  // more row blocks than the grid's y axis holds (a triples tensor has them):
+  // they go on along z, which is free then, because so many tiles are not split
+  constexpr unsigned kMaxY = 65535;
+  const unsigned rows = unsigned((M + kRows - 1) / kRows), splits = unsigned((p.nseg + p.spc - 1) / p.spc);
+  RTCC3_CHECK(rows <= kMaxY || splits == 1, kErrArg, "sliced product: splits of a long output");
+  a.zrow = splits == 1 ? kMaxY : 0;
+  a.zspc = splits == 1 ? 0 : unsigned(p.spc);
+  const dim3 grid(unsigned((2LL * N + p.nt - 1) / p.nt), std::min(rows, kMaxY),
+                  splits == 1 ? (rows + kMaxY - 1) / kMaxY : splits);
 #define RTCC3_OZ(NTV)                                                  \
   if (A.kc && B.kc) launch_nt<NTV, true, true>(a, grid, s);            \
   else if (A.kc) launch_nt<NTV, true, false>(a, grid, s);              \

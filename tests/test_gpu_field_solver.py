@@ -57,3 +57,22 @@ def test_rotated_solver_propagation_fp32_matches_fixed_point():
         out.append(eng.propagate_rk4(0.01, 3)[0])
         eng.close()
     assert _rel(out[0], out[1]) < 1e-5
+
+
+@pytest.mark.parametrize("o,v", [(8, 52), (40, 12)])
+def test_fixed_point_with_more_than_65535_row_blocks(o, v):
+    """Stored FP64 triples whose slot products have o2 v3 (8, 52) and o3 v2
+    (40, 12) rows, more than 65,535 blocks of 128: both solvers agree."""
+    from paper_2407_18947_gb300.api import RTCC3
+    s = make_system(o, v, seed=60 + o)
+    amps = random_amplitudes(o, v, seed=61)
+    out = []
+    for solver in (0, 1):
+        eng = RTCC3(o, v, precision=0, field_solver=solver, triples_chunk=-1)
+        eng.set_hamiltonian(s.eps, s.Lfac, s.dipole)
+        eng.set_field(0, 1, 1e-4, direction=(0.3, 0.0, 1.0))
+        eng.set_amplitudes(0, *amps)
+        out.append(eng.compute_residuals(0, 0.0))
+        eng.close()
+    for k in ("r_t1", "r_t2", "r_l1", "r_l2"):
+        assert _rel(out[1][k], out[0][k]) < 1e-10, k
