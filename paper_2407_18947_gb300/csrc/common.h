@@ -10,6 +10,8 @@
 #include <string>
 #include <vector>
 
+#include "per_device.h"
+
 namespace rtcc3 {
 
 // Complex numbers are interleaved (re, im) pairs: double2 / float2.
@@ -53,6 +55,17 @@ enum Status {
 inline void upload(void* dst, const void* src, size_t bytes) {
   RTCC3_CUDA(cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice));
   RTCC3_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
+}
+
+// Opts a kernel in to more than 48 KB of dynamic shared memory: a setting of
+// the current device only, so it is remembered for each device.
+template <typename K>
+inline void allow_smem(PerDevice& done, K kernel, int bytes) {
+  int dev = 0;
+  RTCC3_CUDA(cudaGetDevice(&dev));
+  done.once(dev, [&] {
+    RTCC3_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  });
 }
 
 // Optional per-kernel timing with CUDA events (eager launches only: CUDA

@@ -541,12 +541,8 @@ void launch_t(const EigJob& a, const EigJob& b, int* status, cudaStream_t s) {
     level = 1;
     smem = (2 * nmax * nmax + nmax) * vs;
   }
-  static bool attr = false;
-  if (!attr) {
-    RTCC3_CUDA(cudaFuncSetAttribute(k_eig_warp<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    int(kMaxSmem)));
-    attr = true;
-  }
+  static PerDevice attr;
+  allow_smem(attr, k_eig_warp<T>, int(kMaxSmem));
   k_eig_refine<T><<<2 * kCl, kRefineThreads, 0, s>>>(a, b);
   RTCC3_CUDA(cudaGetLastError());
   k_eig_warp<T><<<2, 32, smem, s>>>(a, b, level, status);

@@ -22,7 +22,6 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 
 #include "tc_ptx.h"
@@ -642,13 +641,8 @@ k_oz_finish_wide(const double2* __restrict__ part, int nsplit, int M, int N, dou
 template <int NT, bool AKC, bool BKC>
 void launch_nt(const OzArgs& a, dim3 grid, cudaStream_t s) {
   using L = OzSmem<NT>;
-  // per device and process; set again by a second thread without harm
-  static std::atomic<bool> attr{false};
-  if (!attr.load(std::memory_order_acquire)) {
-    RTCC3_CUDA(cudaFuncSetAttribute(k_oz_gemm<NT, AKC, BKC>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal));
-    attr.store(true, std::memory_order_release);
-  }
+  static PerDevice attr;
+  allow_smem(attr, k_oz_gemm<NT, AKC, BKC>, L::kTotal);
   k_oz_gemm<NT, AKC, BKC><<<grid, 32 * kWorkers + 32, L::kTotal, s>>>(a);
   RTCC3_CUDA(cudaGetLastError());
 }

@@ -923,16 +923,9 @@ void launch_short(const CUtensorMap& ma, const CUtensorMap& mb, const TcOperands
                   const long long* cM, const long long* cN, long long coff, float alpha,
                   bool accumulate, int* err, cudaStream_t s) {
   constexpr int BN = TcShortSmem<NACC, true>::BN;
-  static bool attr = false;
-  if (!attr) {
-    RTCC3_CUDA(cudaFuncSetAttribute(k_tc_gemm_short<NACC, true>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    TcShortSmem<NACC, true>::kTotal));
-    RTCC3_CUDA(cudaFuncSetAttribute(k_tc_gemm_short<NACC, false>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    TcShortSmem<NACC, false>::kTotal));
-    attr = true;
-  }
+  static PerDevice attr_acc, attr_over;
+  allow_smem(attr_acc, k_tc_gemm_short<NACC, true>, TcShortSmem<NACC, true>::kTotal);
+  allow_smem(attr_over, k_tc_gemm_short<NACC, false>, TcShortSmem<NACC, false>::kTotal);
   const int nkb = op.Kp / 32, mblocks = (op.M + kBM - 1) / kBM, nblocks = (2 * op.N + BN - 1) / BN;
   long long best = -1;
   int tpc = nblocks;
@@ -1110,12 +1103,8 @@ void launch(const CUtensorMap& ma, const CUtensorMap& mb, const TcOperands& op, 
             const long long* cM, const long long* cN, long long coff, float alpha, bool accumulate,
             int nsplit, float* partial, int* err, cudaStream_t s) {
   using L = TcSmem<BN, SPLIT>;
-  static bool attr = false;
-  if (!attr) {
-    RTCC3_CUDA(cudaFuncSetAttribute(k_tc_gemm<BN, BF16, SPLIT>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal));
-    attr = true;
-  }
+  static PerDevice attr;
+  allow_smem(attr, k_tc_gemm<BN, BF16, SPLIT>, L::kTotal);
   const int Nr = 2 * op.N;
   const int nkb = op.Kp / (128 / op.elem_bytes);
   const int per = (nkb + nsplit - 1) / nsplit;
@@ -1451,14 +1440,9 @@ void launch_direct(const float2* A, long long aoff, const long long* aM, const l
   const int nkb = op.Kp / 32;
   const int per = (nkb + nsplit - 1) / nsplit;
   const int nchains = (nkb + per - 1) / per;
-  static bool attr = false;
-  if (!attr) {
-    RTCC3_CUDA(cudaFuncSetAttribute(k_tc_gemm_direct<BN, true>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal));
-    RTCC3_CUDA(cudaFuncSetAttribute(k_tc_gemm_direct<BN, false>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal));
-    attr = true;
-  }
+  static PerDevice attr_kc, attr_kn;
+  allow_smem(attr_kc, k_tc_gemm_direct<BN, true>, L::kTotal);
+  allow_smem(attr_kn, k_tc_gemm_direct<BN, false>, L::kTotal);
   const long long tiles = (long long)((Nr + BN - 1) / BN) * ((op.M + kBM - 1) / kBM);
   const int cpc = chains_per_cta(tiles, nchains);
   const int zz = (nchains + cpc - 1) / cpc;
@@ -1486,12 +1470,8 @@ bool launch_chains(const void* Atiled, const CUtensorMap& mb, const TcOperands& 
   const int per = (nkb + nsplit - 1) / nsplit;
   const int nchains = (nkb + per - 1) / per;
   if (nchains != nsplit) return false;  // every partial slice must be written
-  static bool attr = false;
-  if (!attr) {
-    RTCC3_CUDA(cudaFuncSetAttribute(k_tc_gemm_chains<BN, BF16, SPLIT>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal));
-    attr = true;
-  }
+  static PerDevice attr;
+  allow_smem(attr, k_tc_gemm_chains<BN, BF16, SPLIT>, L::kTotal);
   const long long tiles = (long long)((Nr + BN - 1) / BN) * ((op.M + kBM - 1) / kBM);
   const int cpc = chains_per_cta(tiles, nchains);
   const int zz = (nchains + cpc - 1) / cpc;
