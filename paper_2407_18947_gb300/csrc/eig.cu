@@ -243,15 +243,17 @@ k_eig_refine(EigJob ja, EigJob jb) {
               if (dl.x * s.x + dl.y * s.y < T(0)) s = X::scale(s, T(-1));
             }
             const V den = X::add(dl, s);
-            e = j > i ? X::scale(X::div(b, den), T(-1)) : X::div(c, den);
-            q = X::sub(q, X::mul(X::div(b, den), X::div(c, den)));
+            const V bd = X::div(b, den), cd = X::div(c, den);
+            e = j > i ? X::scale(bd, T(-1)) : cd;
+            q = X::sub(q, X::mul(bd, cd));
             const T ae = X::abs(e);
             mx = ae > mx || !(ae == ae) ? ae : mx;
           }
         }
         if (it > 0) {
           // Y has to be the inverse of X too
-          const T ar = X::abs(r_at(i, j));
+          const V r = r_at(i, j);
+          const T ar = fabs(r.x) + fabs(r.y);
           mx = ar > mx || !(ar == ar) ? ar : mx;
         }
         W.E[size_t(i) * n + j] = e;
