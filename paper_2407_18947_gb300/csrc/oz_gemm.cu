@@ -454,7 +454,9 @@ __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs 
             if (k < P.K) prefetch_l2(aat(u, 16 * P.aK[k]));
           }
         }
-        if (it >= 2 && ok) ok = mbar_wait(smem_u32(&empty[st]), ((it >> 1) - 1) & 1, P.budget);
+        // (lanes run out of their budgets one by one; what follows takes a whole warp)
+        if (it >= 2)
+          ok = __all_sync(0xffffffffu, ok && mbar_wait(smem_u32(&empty[st]), ((it >> 1) - 1) & 1, P.budget));
         if (ok) {
           const uint32_t sa = smem_u32(smem + st * L::kStage), sb = sa + kSl * L::kASlice;
           if (wact || it < 2) {

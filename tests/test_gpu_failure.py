@@ -81,3 +81,25 @@ def test_checked_mode_finds_no_overrun_and_gives_the_same_result():
         out.append(np.asarray(eng.propagate_rk4(0.01, 2)[0]))
         eng.close()
     assert np.abs(out[0] - out[1]).max() < 1e-9
+
+
+def test_sliced_product_wait_budget_reports_timeout_and_context_recovers():
+    """FP64: the sliced products wait for their own pipeline too."""
+    from paper_2407_18947_gb300._lib import ERR_TIMEOUT, RTCC3Error
+    s = make_system(8, 16, seed=82)
+    ref_eng = _engine(s, 0)
+    ref = _run(ref_eng)
+    ref_eng.set_profiling(True)
+    _run(ref_eng)
+    assert ref_eng.kernel_stats()["contract_sliced_c128"]["launches"] > 0
+    ref_eng.close()
+    eng = _engine(s, 0)
+    eng.set_wait_budgets(1, 0)
+    with pytest.raises(RTCC3Error) as ei:
+        _run(eng)
+    assert ei.value.code == ERR_TIMEOUT and "tensor-core" in str(ei.value)
+    eng.set_wait_budgets(0, 0)
+    for _ in range(2):
+        got = _run(eng)
+        assert np.abs(got - ref).max() <= 1e-12 * np.abs(ref).max()
+    eng.close()
