@@ -561,12 +561,14 @@ void final_observables(rtcc3_ctx* ctx, const std::vector<int>& sweeps) {
 template <typename R>
 void check_device_timeout(rtcc3_ctx* ctx) {
   Engine<R>& E = ctx->run<R>().E;
-  int flag = 0;
-  RTCC3_CUDA(cudaMemcpy(&flag, E.error_flag(), sizeof(int), cudaMemcpyDeviceToHost));
-  if (flag) {
-    RTCC3_CUDA(cudaMemset(E.error_flag(), 0, sizeof(int)));
+  int flags[2] = {};
+  RTCC3_CUDA(cudaMemcpy(flags, E.error_flag(), sizeof(flags), cudaMemcpyDeviceToHost));
+  if (flags[0] || flags[1]) {
+    RTCC3_CUDA(cudaMemset(E.error_flag(), 0, sizeof(flags)));
     RTCC3_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
-    if (flag & kEigStatusBase) {
+    // a wait that gave up may be what spoiled a matrix: it is reported first
+    if (!flags[1]) {
+      const int flag = flags[0];
       const int reason = (flag >> 20) & 0xf, n = (flag >> 10) & 0x3ff, row = flag & 0x3ff;
       throw Error(reason == kEigNonFinite ? RTCC3_ERR_NONFINITE : RTCC3_ERR_TIMEOUT,
                   std::string("field eigensolver (order ") + std::to_string(n) + "): " +
@@ -963,10 +965,11 @@ void triples_noalloc_impl(rtcc3_ctx* ctx, int b, double time, const double2* t1,
   // the engine's host-side tables must outlive the copies it enqueued
   RTCC3_CUDA(cudaStreamSynchronize(st));
   if (E.tensor_cores() || ctx->fp64()) {
-    int flag = 0;
-    RTCC3_CUDA(cudaMemcpy(&flag, E.error_flag(), sizeof(int), cudaMemcpyDeviceToHost));
-    // FP64: only a tensor-core wait (the eigensolver's codes stay in the result)
-    RTCC3_CHECK(flag == 0 || (ctx->fp64() && (flag & kEigStatusBase)), RTCC3_ERR_TIMEOUT, "a tensor-core kernel gave up waiting on its pipeline");
+    int flags[2] = {};
+    RTCC3_CUDA(cudaMemcpy(flags, E.error_flag(), sizeof(flags), cudaMemcpyDeviceToHost));
+    // (in FP64 a failed eigenbasis stays in the result)
+    RTCC3_CHECK(!flags[1] && (ctx->fp64() || !flags[0]), RTCC3_ERR_TIMEOUT,
+                "a tensor-core kernel gave up waiting on its pipeline");
   }
 }
 

@@ -1079,11 +1079,11 @@ template <typename R>
 int* Engine<R>::error_flag() {
   if (!err_) {
     if (pool_) {
-      err_ = static_cast<int*>(pool_->take(sizeof(int)));
-      RTCC3_CUDA(cudaMemsetAsync(err_, 0, sizeof(int), stream_));
+      err_ = static_cast<int*>(pool_->take(2 * sizeof(int)));
+      RTCC3_CUDA(cudaMemsetAsync(err_, 0, 2 * sizeof(int), stream_));
     } else {
-      RTCC3_CUDA(cudaMalloc(&err_, sizeof(int)));
-      RTCC3_CUDA(cudaMemset(err_, 0, sizeof(int)));
+      RTCC3_CUDA(cudaMalloc(&err_, 2 * sizeof(int)));
+      RTCC3_CUDA(cudaMemset(err_, 0, 2 * sizeof(int)));
       RTCC3_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
     }
   }
@@ -1774,7 +1774,7 @@ void Engine<R>::run_contract_tc(ContractPlan& P, double alpha, const C* pa, cons
     if (P.tc_nsplit > 1)
       part = static_cast<float*>(
           scratch(tc_slot_ + 2, size_t(P.tc_nsplit) * op.M * 2 * op.N * sizeof(float)));
-    int* err = error_flag();
+    int* err = wait_flag();
     const bool a_kc = sw ? P.b_kcontig : P.a_kcontig;
     const double rows_packed = direct ? 2.0 * op.N : op.M + 2.0 * op.N;
     int pk = pbegin();
@@ -1821,7 +1821,7 @@ void Engine<R>::run_contract_oz(ContractPlan& P, double alpha, const C* pa, cons
     C* part = nullptr;
     if (P.oz.nsplit > 1)
       part = static_cast<C*>(scratch(split_slot_, size_t(P.oz.nsplit) * P.M * P.N * sizeof(C)));
-    int* err = error_flag();
+    int* err = wait_flag();
     const int pk = pbegin();
     launches_ += oz_gemm(P.oz, sw ? b : a, sw ? a : b, Mg, Ng, P.K, pc, P.c_off0, sw ? P.cN : P.cM,
                          sw ? P.cM : P.cN, P.c_unit_m != sw, alpha, accumulate, part, err,

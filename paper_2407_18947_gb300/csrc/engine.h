@@ -295,8 +295,11 @@ class Engine {
   // Contractions recorded while the region is open (and their adjoints) may
   // take the tensor-core route; everything else stays on CUDA cores in FP32.
   void set_tc_region(bool open) { tc_region_ = open; }
-  // Device word raised by a bounded wait that gave up (tensor-core kernel).
+  // Two device words: [0] the eigensolver's status (eig_status), [1] raised by
+  // a bounded wait that gave up (tensor-core kernels).  Apart, so that neither
+  // hides the other.
   int* error_flag();
+  int* wait_flag() { return error_flag() + 1; }
   // Clock cycles a tensor-core kernel's wait on another warp may spin before
   // it gives up and raises the error flag (0: the kernels' default).
   // Checked mode: every tensor gets a canary after it, verified (raising

@@ -103,3 +103,23 @@ def test_sliced_product_wait_budget_reports_timeout_and_context_recovers():
         got = _run(eng)
         assert np.abs(got - ref).max() <= 1e-12 * np.abs(ref).max()
     eng.close()
+
+
+@pytest.mark.parametrize("precision", [0, 2])
+def test_wait_that_gave_up_is_not_hidden_by_the_eigensolver(precision):
+    """Both give up in one evaluation: the eigensolver's code leaves the
+    wait's alone, and the wait, which may have spoiled the matrix, is named."""
+    from paper_2407_18947_gb300._lib import ERR_TIMEOUT, RTCC3Error
+    s = make_system(8, 16, seed=83)
+    eng = _engine(s, precision)
+    eng.set_wait_budgets(1, 1)
+    with pytest.raises(RTCC3Error) as ei:
+        _run(eng)
+    assert ei.value.code == ERR_TIMEOUT and "tensor-core" in str(ei.value)
+    eng.set_wait_budgets(0, 1)
+    with pytest.raises(RTCC3Error) as ei:
+        _run(eng)
+    assert ei.value.code == ERR_TIMEOUT and "QR sweeps" in str(ei.value)
+    eng.set_wait_budgets(0, 0)
+    assert np.isfinite(_run(eng)).all()
+    eng.close()
