@@ -562,10 +562,9 @@ template <typename R>
 void check_device_timeout(rtcc3_ctx* ctx) {
   Engine<R>& E = ctx->run<R>().E;
   int flags[2] = {};
-  RTCC3_CUDA(cudaMemcpy(flags, E.error_flag(), sizeof(flags), cudaMemcpyDeviceToHost));
+  E.read_flags(flags);
   if (flags[0] || flags[1]) {
-    RTCC3_CUDA(cudaMemset(E.error_flag(), 0, sizeof(flags)));
-    RTCC3_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
+    E.clear_flags();
     // a wait that gave up may be what spoiled a matrix: it is reported first
     if (!flags[1]) {
       const int flag = flags[0];
@@ -578,6 +577,15 @@ void check_device_timeout(rtcc3_ctx* ctx) {
     }
     throw Error(RTCC3_ERR_TIMEOUT, "a tensor-core pipeline wait gave up");
   }
+}
+
+// The same for the calls in which a failed eigenbasis stays in the result: a
+// wait that gave up does not.
+template <typename R>
+void check_waits(rtcc3_ctx* ctx) {
+  int flags[2] = {};
+  ctx->run<R>().E.read_flags(flags);
+  if (flags[1]) check_device_timeout<R>(ctx);
 }
 
 void drop_graph(rtcc3_ctx* ctx) {
@@ -801,6 +809,7 @@ void ground_state_impl(rtcc3_ctx* ctx, double tol, int maxiter) {
       RTCC3_CUDA(cudaMemcpyAsync(&mx, ctx->maxr, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
       RTCC3_CUDA(cudaMemcpyAsync(d.data(), dots, mm * sizeof(double2), cudaMemcpyDeviceToHost, ctx->stream));
       RTCC3_CUDA(cudaStreamSynchronize(ctx->stream));
+      check_waits<R>(ctx);
       ctx->gs_history.push_back(mx);
       if (!lam) ctx->gs_t_iters = int(ctx->gs_history.size());
       if (!std::isfinite(mx)) {
@@ -880,6 +889,7 @@ void triples_impl(rtcc3_ctx* ctx, int b, double time, const double2* t1, const d
     launch_export<R>(E.data(S.r2), x2, n2, ctx->stream);
   }
   RTCC3_CUDA(cudaStreamSynchronize(ctx->stream));
+  check_waits<R>(ctx);
 }
 
 // ---- allocation-free triples map ------------------------------------------
@@ -966,7 +976,7 @@ void triples_noalloc_impl(rtcc3_ctx* ctx, int b, double time, const double2* t1,
   RTCC3_CUDA(cudaStreamSynchronize(st));
   if (E.tensor_cores() || ctx->fp64()) {
     int flags[2] = {};
-    RTCC3_CUDA(cudaMemcpy(flags, E.error_flag(), sizeof(flags), cudaMemcpyDeviceToHost));
+    E.read_flags(flags);
     // (in FP64 a failed eigenbasis stays in the result)
     RTCC3_CHECK(!flags[1] && (ctx->fp64() || !flags[0]), RTCC3_ERR_TIMEOUT,
                 "a tensor-core kernel gave up waiting on its pipeline");

@@ -1046,7 +1046,7 @@ Engine<R>::~Engine() {
     if (kv.second->dev) cudaFree(kv.second->dev);
   for (int s = 0; s < kScratchSlots; ++s)
     if (scratch_[s]) cudaFree(scratch_[s]);
-  if (err_) cudaFree(err_);
+  if (err_host_) cudaFreeHost(const_cast<int*>(err_host_));
 }
 
 template <typename R>
@@ -1082,12 +1082,31 @@ int* Engine<R>::error_flag() {
       err_ = static_cast<int*>(pool_->take(2 * sizeof(int)));
       RTCC3_CUDA(cudaMemsetAsync(err_, 0, 2 * sizeof(int), stream_));
     } else {
-      RTCC3_CUDA(cudaMalloc(&err_, 2 * sizeof(int)));
-      RTCC3_CUDA(cudaMemset(err_, 0, 2 * sizeof(int)));
-      RTCC3_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
+      void *h = nullptr, *dev = nullptr;
+      RTCC3_CUDA(cudaHostAlloc(&h, 2 * sizeof(int), cudaHostAllocMapped));
+      err_host_ = static_cast<int*>(h);
+      err_host_[0] = err_host_[1] = 0;
+      RTCC3_CUDA(cudaHostGetDevicePointer(&dev, h, 0));
+      err_ = static_cast<int*>(dev);
     }
   }
   return err_;
+}
+
+template <typename R>
+void Engine<R>::read_flags(int* out) {
+  int* dev = error_flag();
+  if (pool_) {
+    RTCC3_CUDA(cudaMemcpy(out, dev, 2 * sizeof(int), cudaMemcpyDeviceToHost));
+    return;
+  }
+  out[0] = err_host_[0];
+  out[1] = err_host_[1];
+}
+
+template <typename R>
+void Engine<R>::clear_flags() {
+  if (err_host_) err_host_[0] = err_host_[1] = 0;
 }
 
 template <typename R>

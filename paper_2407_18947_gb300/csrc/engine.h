@@ -300,6 +300,11 @@ class Engine {
   // hides the other.
   int* error_flag();
   int* wait_flag() { return error_flag() + 1; }
+  // Both words into out[2] (the streams that may raise them have been waited
+  // for).  They live in pinned host memory, so that looking costs no copy (a
+  // copy and its wait: 8 us of a 1 ms call), or in the caller's pool.
+  void read_flags(int* out);
+  void clear_flags();
   // Clock cycles a tensor-core kernel's wait on another warp may spin before
   // it gives up and raises the error flag (0: the kernels' default).
   // Checked mode: every tensor gets a canary after it, verified (raising
@@ -459,6 +464,7 @@ class Engine {
   int eig_cap_ = 0;
   bool tc_region_ = false;
   int* err_ = nullptr;
+  volatile int* err_host_ = nullptr;  // the same words, unless in a pool
   cudaStream_t side_ = nullptr;
   cudaEvent_t fork_ev_ = nullptr, join_ev_ = nullptr;
   DevicePool* pool_ = nullptr;

@@ -123,3 +123,41 @@ def test_wait_that_gave_up_is_not_hidden_by_the_eigensolver(precision):
     eng.set_wait_budgets(0, 0)
     assert np.isfinite(_run(eng)).all()
     eng.close()
+
+
+@pytest.mark.parametrize("precision", [2, 0])
+def test_triples_entry_points_report_a_wait_that_gave_up(precision):
+    import torch
+    from paper_2407_18947_gb300._lib import ERR_TIMEOUT, RTCC3Error
+    from paper_2407_18947_gb300.autograd import TriplesResidual
+    s = make_system(8, 16, seed=84)
+    eng = _engine(s, precision)
+    t1, t2, u1, u2 = (torch.tensor(x, device="cuda")
+                      for x in random_amplitudes(s.nocc, s.nvir, seed=85))
+    t1.requires_grad_(True)
+    t2.requires_grad_(True)
+    ref = [x.detach() for x in TriplesResidual.apply(t1, t2, eng, 0, 0.1)]
+    eng.set_wait_budgets(1, 0)
+    with pytest.raises(RTCC3Error) as ei:
+        TriplesResidual.apply(t1, t2, eng, 0, 0.1)
+    assert ei.value.code == ERR_TIMEOUT and "tensor-core" in str(ei.value)
+    eng.set_wait_budgets(0, 0)
+    x = TriplesResidual.apply(t1, t2, eng, 0, 0.1)
+    for a, b in zip(x, ref):
+        assert (a - b).abs().max() <= 1e-6 * b.abs().max()
+    eng.set_wait_budgets(1, 0)
+    with pytest.raises(RTCC3Error) as ei:
+        torch.autograd.grad(x, [t1, t2], [u1, u2])
+    assert ei.value.code == ERR_TIMEOUT and "tensor-core" in str(ei.value)
+    eng.close()
+
+
+@pytest.mark.parametrize("precision", [2, 0])
+def test_ground_state_reports_a_wait_that_gave_up(precision):
+    from paper_2407_18947_gb300._lib import ERR_TIMEOUT, RTCC3Error
+    eng = _engine(make_system(8, 16, seed=86), precision)
+    eng.set_wait_budgets(1, 0)
+    with pytest.raises(RTCC3Error) as ei:
+        eng.solve_ground_state(1e-30, 2)
+    assert ei.value.code == ERR_TIMEOUT and "tensor-core" in str(ei.value)
+    eng.close()
