@@ -1838,7 +1838,7 @@ void Engine<R>::run_contract_oz(ContractPlan& P, double alpha, const C* pa, cons
     const OzOperand a{pa, P.a_off0, P.aM, P.aK, P.a_kcontig}, b{pb, P.b_off0, P.bN, P.bK, P.b_kcontig};
     const int Mg = sw ? P.N : P.M, Ng = sw ? P.M : P.N;
     C* part = nullptr;
-    if (P.oz.nsplit > 1)
+    if (P.oz.nseg > 1)
       part = static_cast<C*>(scratch(split_slot_, size_t(P.oz.nsplit) * P.M * P.N * sizeof(C)));
     int* err = wait_flag();
     const int pk = pbegin();

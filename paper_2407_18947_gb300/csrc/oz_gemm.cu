@@ -77,13 +77,6 @@ __device__ __forceinline__ void tmem_ld(uint32_t t, uint32_t (&r)[4]) {
                : "r"(t));
 }
 
-__device__ __forceinline__ void tmem_ld(uint32_t t, uint32_t (&r)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                 "=r"(r[7])
-               : "r"(t));
-}
-
 // |x| as a sortable word whose top 11 bits are its exponent field.
 __device__ __forceinline__ uint32_t hiabs(uint32_t hi) { return hi & 0x7fffffffu; }
 
@@ -252,14 +245,15 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 struct OzArgs {
   const double2 *A, *B;
   const long long *aM, *aK, *bN, *bK, *cM, *cN;
-  double2* C;      // already moved by its offset; the partials when nsplit > 1
+  double2* C;      // already moved by its offset
+  double2* part;   // running sums over a CTA's segments, [split][n][m] (nseg > 1)
   int M, N, K;
   unsigned zrow, zspc;  // row blocks and segments a step of blockIdx.z stands for (one is 0)
   int seg, nseg, spc;
   int ash;         // alpha = (neg ? -1 : 1) 2^ash alpha_rest, neg = all ones or 0
   uint32_t neg;
   double alpha_rest;
-  int accumulate, to_part, c_m;
+  int accumulate, splits, c_m;
   int* err;
   long long budget;
 };
@@ -269,7 +263,7 @@ __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs 
   using L = OzSmem<NT>;
   constexpr int NB = NT / 2;   // complex columns
   constexpr int CPT = NT / 4;  // real columns a worker thread reads back
-  constexpr int CU = CPT % 8 == 0 ? 8 : 4;  // at a time
+  constexpr int CU = 4;        // at a time (eight spill)
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::kBarOff);
@@ -299,7 +293,7 @@ __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs 
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tmem_slot)), "r"(L::kCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  } else if (!P.to_part) {
+  } else if (P.splits == 1) {
     if (tid < kRows) sCM[tid] = m0 + tid < P.M ? P.cM[m0 + tid] : 0;
     else if (tid < kRows + NB) sCN[tid - kRows] = n0 + tid - kRows < P.N ? P.cN[n0 + tid - kRows] : 0;
   }
@@ -493,11 +487,15 @@ __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs 
       if (ok) ok = mbar_wait(smem_u32(done), (sg - s0) & 1, P.budget);
       ok = __all_sync(0xffffffffu, ok);
       const int q = w & 3, c0 = (w >> 2) * CPT;
-      // a staged tile overwrites the stages: every MMA has completed, and no
-      // warp converts any more (a staged tile is its CTA's only segment)
+      // The CTA's segments are summed here, between segments in global memory
+      // (read back from L2 by the thread that wrote it).  The sum of the last one
+      // is staged where the stages were: every MMA has completed, and no warp
+      // converts any more.
+      const bool more = sg > s0, stage = sg + 1 == s1 && P.splits == 1;
       double* stg = reinterpret_cast<double*>(smem) + (q * 32 + lane) * (2 * L::kPitch) + c0;
       const int m = m0 + q * 32 + lane;
-      double2* prow = P.C + ((long long)sg * P.M + m) * P.N + n0 + (c0 >> 1);
+      const int ncol = min(NB, P.N - n0) - (c0 >> 1);
+      double2* prow = P.part + ((long long)(P.zspc ? blockIdx.z : 0) * P.N + n0 + (c0 >> 1)) * P.M + m;
       if (ok && m0 + q * 32 < P.M && 2 * n0 + c0 < 2 * P.N) {  // else: no output here
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const int F = eA[q * 32 + lane] - 2112 + P.ash;
@@ -520,15 +518,19 @@ __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs 
               for (int g = 0; g < kSl; ++g) x[g] = __uint_as_float(v[g][j + i]);
               d[i] = join(x, F + eB[(c0 + cc + j) >> 1], P.neg);
             }
-            const double2 z = make_double2(d[0], d[1]);
-            if (!P.to_part) *reinterpret_cast<double2*>(stg + cc + j) = z;
-            else if (m < P.M && n0 + ((c0 + cc + j) >> 1) < P.N) prow[(cc + j) >> 1] = z;
+            double2 z = make_double2(d[0], d[1]);
+            if (more) {
+              const double2 o = m < P.M && ((cc + j) >> 1) < ncol ? prow[(long long)((cc + j) >> 1) * P.M] : zero;
+              z.x += o.x; z.y += o.y;
+            }
+            if (stage) *reinterpret_cast<double2*>(stg + cc + j) = z;
+            else if (m < P.M && ((cc + j) >> 1) < ncol) prow[(long long)((cc + j) >> 1) * P.M] = z;
           }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       }
     }
-    if (!P.to_part) {
+    if (P.splits == 1) {
       // ---- write the tile from shared memory along C's contiguous index
       asm volatile("bar.sync 1, %0;" ::"r"(32 * kWorkers) : "memory");
       const double2* sc = reinterpret_cast<const double2*>(smem);
@@ -575,7 +577,7 @@ __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs 
   }
 }
 
-// C (+)= alpha sum_s part[s][m][n], the splits in a fixed order: LS lanes of a
+// C (+)= alpha sum_s part[s][n][m], the splits in a fixed order: LS lanes of a
 // warp share one output (every LS-th split each, joined by shuffles).
 template <int LS>
 __global__ void __launch_bounds__(256)
@@ -601,7 +603,7 @@ k_oz_finish(const double2* __restrict__ part, int nsplit, int M, int N, double2*
     si += __shfl_xor_sync(0xffffffffu, si, d);
   }
   if (t >= total || lane >= PO) return;
-  const long long idx = cM[t / N] + cN[t % N];
+  const long long idx = cM[t % M] + cN[t / M];
   double2 v = make_double2(alpha * sr, alpha * si);
   if (accumulate) { v.x += C[idx].x; v.y += C[idx].y; }
   C[idx] = v;
@@ -634,7 +636,7 @@ k_oz_finish_wide(const double2* __restrict__ part, int nsplit, int M, int N, dou
     }
   }
   if (threadIdx.x >= 4 || t >= total) return;
-  const long long idx = cM[t / N] + cN[t % N];
+  const long long idx = cM[t % M] + cN[t / M];
   double2 v = make_double2(alpha * red[o].x, alpha * red[o].y);
   if (accumulate) { v.x += C[idx].x; v.y += C[idx].y; }
   C[idx] = v;
@@ -666,9 +668,10 @@ OzPlan oz_plan(long long M, long long N, long long K) {
       long long nseg = (K + seg - 1) / seg;
       seg = ((K + nseg - 1) / nseg + 7) / 8 * 8;
       nseg = (K + seg - 1) / seg;
-      // CTAs: one per SM is resident; with several segments each has its own
-      // partial sum, and a CTA takes several of them in turn once the tiles
-      // fill two waves
+      // CTAs: one per SM is resident; a CTA takes several segments in turn and
+      // sums them once the tiles fill two waves.  So the running sums are one
+      // per output, or at most 304 tiles of them (20 MB): a partial sum per
+      // segment was v / 128 of a triples tensor, 4.5 GB at (15, 57).
       long long zs = std::min(nseg, std::max<long long>(1, (2 * 152) / tiles));
       const long long spc = (nseg + zs - 1) / zs;
       zs = (nseg + spc - 1) / spc;
@@ -678,14 +681,15 @@ OzPlan oz_plan(long long M, long long N, long long K) {
       const double per = 14000.0 + double((seg + 7) / 8) * (1500.0 + 8.0 * nt) + 60.0 * nt;
       const double waves = std::ceil(double(tiles * zs) / slots);
       double cost = waves * double(spc) * per + 6000.0;
-      if (nseg > 1) cost += 6000.0 + double(nseg) * double(M) * double(N) / slots;
+      if (spc > 1) cost += waves * double(spc) * 70.0 * nt;  // the adds
+      if (zs > 1) cost += 6000.0 + double(zs) * double(M) * double(N) / slots;
       if (cost < best.cost) {
         best.swap = sw != 0;
         best.nt = nt;
         best.seg = int(seg);
         best.nseg = int(nseg);
         best.spc = int(spc);
-        best.nsplit = int(nseg);
+        best.nsplit = int(zs);
         best.cost = cost;
       }
     }
@@ -715,10 +719,11 @@ int oz_gemm(const OzPlan& p, const OzOperand& A, const OzOperand& B, int M, int 
   a.budget = wait_budget > 0 ? wait_budget : kWaitBudget;
   a.alpha_rest = 1.0;
   const bool split = p.nsplit > 1;
-  a.to_part = split ? 1 : 0;
+  a.splits = p.nsplit;
   a.accumulate = !split && accumulate ? 1 : 0;
   a.c_m = !split && c_m ? 1 : 0;
-  a.C = split ? part : C + coff;
+  a.C = C + coff;
+  a.part = part;
   if (!split) {
     // alpha as a sign, a power of two (joined without FP64 work) and the rest
     int e = 0;
@@ -733,7 +738,7 @@ int oz_gemm(const OzPlan& p, const OzOperand& A, const OzOperand& B, int M, int 
   // more row blocks than the grid's y axis holds (a triples tensor has them):
   // they go on along z, which is free then, because so many tiles are not split
   constexpr unsigned kMaxY = 65535;
-  const unsigned rows = unsigned((M + kRows - 1) / kRows), splits = unsigned((p.nseg + p.spc - 1) / p.spc);
+  const unsigned rows = unsigned((M + kRows - 1) / kRows), splits = unsigned(p.nsplit);
   RTCC3_CHECK(rows <= kMaxY || splits == 1, kErrArg, "sliced product: splits of a long output");
   a.zrow = splits == 1 ? kMaxY : 0;
   a.zspc = splits == 1 ? 0 : unsigned(p.spc);

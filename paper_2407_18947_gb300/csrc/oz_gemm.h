@@ -23,7 +23,8 @@ namespace rtcc3 {
 
 // How one contraction runs: which operand takes the 128-row side (swap:
 // the plan's B), the real columns per tile, the K segments (complex elements
-// per segment, segments per CTA) and the number of partial sums.
+// per segment, segments per CTA) and the number of CTAs that share a tile's
+// segments, each with its own sum.
 struct OzPlan {
   bool swap = false;
   int nt = 64;
@@ -41,9 +42,9 @@ struct OzOperand {
   bool kc = false;                                 // contiguous along k
 };
 
-// C[coff + cM[m] + cN[n]] (+)= alpha sum_k A[m,k] B[n,k]; with p.nsplit > 1
-// the partial sums go to part (nsplit x M x N) and a second launch adds them
-// in a fixed order.  c_m: C's contiguous index is on the A side.  Returns the
+// C[coff + cM[m] + cN[n]] (+)= alpha sum_k A[m,k] B[n,k]; with p.nseg > 1 the
+// sums of successive segments go through part (nsplit x N x M), with p.nsplit
+// > 1 a second launch adds the CTAs' sums in a fixed order.  c_m: C's contiguous index is on the A side.  Returns the
 // number of kernel launches.
 int oz_gemm(const OzPlan& p, const OzOperand& A, const OzOperand& B, int M, int N, int K, double2* C,
             long long coff, const long long* cM, const long long* cN, bool c_m, double alpha,
