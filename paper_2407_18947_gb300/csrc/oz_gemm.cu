@@ -12,11 +12,12 @@
 //
 // No FP64 instruction is used on the way to a first result: conversion and
 // joining are integer work, because an SM has 64 times fewer FP64 lanes than
-// integer ones.  The code is kept small (rolled loops): fetched once per tile,
+// integer ones.  FP64 sums again what fixed point cannot hold as accurately
+// (settle).  The code is kept small (rolled loops): fetched once per tile,
 // 85 KB of straight-line code took longer than the work.  Bound by the
 // integer work and load latencies (3800 x 14440 x 48: 52000 warp instructions
 // and 31000 clocks per tile, of which the MMAs take 7000; 17.6 ms on the FP64
-// cores, 1.35 ms here).
+// cores, 1.48 ms here, 0.12 of them for the test that settle() needs).
 #include "oz_gemm.h"
 
 #include <cuda_fp16.h>
@@ -35,7 +36,8 @@ constexpr int kRows = 128;          // A rows per tile
 constexpr int kKC = 16;             // complex k per stage (64-byte FP16 rows)
 constexpr int kWorkers = 16;        // worker warps
 constexpr int kSegMax = 128;        // complex k per segment (256 real: see oz_gemm.h; a power of two)
-constexpr unsigned long long kBias = 0x8080808080808080ULL;
+
+constexpr int kWPitch = 48;         // bytes between the weights of two rows (32 each, no bank conflicts)
 
 template <int NT>
 struct OzSmem {
@@ -45,7 +47,9 @@ struct OzSmem {
   static constexpr int kBarOff = 2 * kStage;
   static constexpr int kExpOff = kBarOff + 64;  // row exponents, two segments
   static constexpr int kTabOff = kExpOff + 2 * (kRows + 32) * 4;  // k offsets (two segments), output offsets
-  static constexpr int kTotal = kTabOff + (4 * kSegMax + kRows + NT / 2) * 8 + 1024;
+  static constexpr int kWOff = kTabOff + (4 * kSegMax + kRows + NT / 2) * 8;  // weights of the rows' elements
+  static constexpr int kRowOff = kWOff + (kRows + 32) * kWPitch;  // offsets of the rows
+  static constexpr int kTotal = kRowOff + (kRows + 32) * 8 + 1024;
   static constexpr int kCols = NT <= 16 ? 128 : (NT <= 32 ? 256 : 512);  // TMEM columns (a power of two)
   static_assert(kRows * kPitch * 16 <= 2 * kStage, "output staging");
   static_assert(kTotal <= 232448, "shared memory per CTA");
@@ -81,16 +85,18 @@ __device__ __forceinline__ void tmem_ld(uint32_t t, uint32_t (&r)[4]) {
 __device__ __forceinline__ uint32_t hiabs(uint32_t hi) { return hi & 0x7fffffffu; }
 
 // |a| (below 2^(F - 1022), F >= 64) as the biased digits of its 62-bit
-// fixed-point form: byte 7 - s is digit s of |a| plus 128.  Elements below
-// 2^-62 of the bound (zeros and subnormals among them) have zero digits.
+// fixed-point form, rounded to nearest: byte 7 - s is digit s of |a| plus 128.
+// Elements below 2^-63 of the bound (zeros and subnormals among them) have zero
+// digits.  The bias of the lower digits and the rounding are added one bit
+// further left; the shift back brings in the first digit's bias.
 __device__ __forceinline__ void digits(double a, int F, uint32_t& yh, uint32_t& yl) {
   const uint32_t hi = uint32_t(__double2hiint(a)), lo = uint32_t(__double2loint(a));
   const int n = min(F - int(hiabs(hi) >> 20), 63);
   const unsigned long long m =
       (static_cast<unsigned long long>((hi & 0xfffffu) | 0x100000u) << 32) | lo;
-  const unsigned long long y = ((m << 9) >> n) + kBias;
-  yh = uint32_t(y >> 32);
-  yl = uint32_t(y);
+  const unsigned long long t = ((m << 10) >> n) + 0x0101010101010101ULL;
+  yh = __funnelshift_r(uint32_t(t >> 32), 1u, 1);
+  yl = __funnelshift_r(uint32_t(t), uint32_t(t >> 32), 1);
 }
 
 // The eight digits of a complex number as pairs of halves (re, im), signs
@@ -159,6 +165,7 @@ __device__ __forceinline__ void store_b(uint32_t addr, const DigitPairs& d, cons
 
 constexpr int kZeroExp = 1 << 16;  // row exponent that makes every digit zero
 constexpr int kNanExp = 1 << 18;  // exponent of a row with a non-finite element
+constexpr int kNullRow = -(1 << 16);  // exponent of a row of zeros (E below half of it: the sum is 0)
 
 __device__ __forceinline__ double join_rare(uint32_t w2, uint32_t w1, uint32_t w0, int e, uint32_t sign) {
   if (e >= kNanExp / 2) return __longlong_as_double(0x7ff8000000000000LL);
@@ -193,9 +200,14 @@ __device__ __forceinline__ uint32_t magnitude(long long hi, long long lo, uint32
 }
 
 // join() of any accumulators: above 2^22, zero sums, results outside the
-// normal range, rows with a non-finite element.
+// normal range, rows with a non-finite element (NaN).  The sums i + j >= 5 are
+// not exact beyond 2^24; that needs digits of nearly the largest size and one
+// sign in four fifths of all terms, which leave more than 0.6 2^24 at the end:
+// NaN too.
 __device__ __noinline__ double join_any(float v0, float v1, float v2, float v3, float v4, float v5,
                                         float v6, float v7, int E, uint32_t sgn) {
+  if (fmaxf(fmaxf(fabsf(v5), fabsf(v6)), fabsf(v7)) >= 10066329.0f)
+    return __longlong_as_double(0x7ff8000000000000LL);
   auto iv = [](float v) { return (long long)__float2int_rn(v); };
   uint32_t w2, w1, w0;
   const uint32_t s = magnitude((iv(v0) << 24) + (iv(v1) << 16) + (iv(v2) << 8) + iv(v3),
@@ -252,11 +264,99 @@ struct OzArgs {
   int seg, nseg, spc;
   int ash;         // alpha = (neg ? -1 : 1) 2^ash alpha_rest, neg = all ones or 0
   uint32_t neg;
-  double alpha_rest;
+  double alpha_rest, alpha_joined;  // alpha_joined = (neg ? -1 : 1) 2^ash
   int accumulate, splits, c_m;
   int* err;
   long long budget;
 };
+
+// Fixed point holds an element to a fraction of its row's largest, so a sum all
+// of whose terms are small beside the product of the two rows' largest elements
+// (rows graded in opposite directions, a row of the identity) would lose digits
+// that FP64 arithmetic keeps.  With |a| <= 2^A, |b| <= 2^B and K complex terms a
+// joined sum is off by at most 2 K (1 + 7.02) 2^-62 2^(A + B) in its real and
+// imaginary parts (two roundings of half a unit of 2^-62, the products i + j >= 8
+// left out), FP64 arithmetic by up to 2 K 2^-53 s, s = sum |a||b|.  So a sum is as
+// accurate as that if s >= 2^-6 2^(A + B).  It is if the result has that size, or
+// if the first 32 terms add up to it by their elements' weights (each 2^-16
+// 2^(A + B) times the two weights); in dense products less than one in a thousand
+// has neither.  Every other output is summed again here in FP64, and so are those
+// whose rows have infinities or NaN, whose digit sums were not exact or whose
+// scale is so small that a component below the normal range counts: they come
+// out as they do in FP64 arithmetic.
+constexpr int kSoundField = 1085;           // exponent field of 2^-6 2^(A + B) less E
+constexpr uint32_t kSoundWeight = 1u << 10;  // the same in products of weights
+
+// Bit j of todo: output z[j stride] of this lane's row lacks this segment's sum.
+// Four outputs at a time, eight lanes each; bound by the FP64 pipe where many are
+// left (8112 x 52 x 52 with a near-identity matrix, a tenth of its outputs: 28 us
+// without, 79 with), by one round's latency where a few are.
+__device__ __forceinline__ void settle(const OzArgs& P, uint32_t todo, double2* z, long long stride,
+                                       const long long* am, const long long* bn, const long long* tk, int klen) {
+  const int lane = threadIdx.x & 31, g = lane >> 3;
+#pragma unroll 1
+  while (const uint32_t lanes = __ballot_sync(0xffffffffu, todo != 0)) {
+    uint32_t t = lanes;
+    int r = -1;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (u == g) r = __ffs(t) - 1;
+      t &= t - 1;
+    }
+    const int mine = __ffs(todo) - 1, j = __shfl_sync(0xffffffffu, mine, r & 31);
+    double sr = 0.0, si = 0.0;
+    if (r >= 0) {
+      const char* pa = reinterpret_cast<const char*>(P.A + am[r]);
+      const char* pb = reinterpret_cast<const char*>(P.B + bn[j]);
+#pragma unroll 1
+      for (int k0 = 0; k0 < klen; k0 += 32) {
+        double2 a[4], b[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int k = k0 + 8 * u + (lane & 7);
+          a[u] = b[u] = make_double2(0.0, 0.0);
+          if (k < klen) {
+            a[u] = *reinterpret_cast<const double2*>(pa + tk[k]);
+            b[u] = *reinterpret_cast<const double2*>(pb + tk[kSegMax + k]);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (k0 + 8 * u < klen) {
+            sr = fma(-a[u].y, b[u].y, fma(a[u].x, b[u].x, sr));
+            si = fma(a[u].y, b[u].x, fma(a[u].x, b[u].y, si));
+          }
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int d = 4; d > 0; d >>= 1) {
+      sr += __shfl_xor_sync(0xffffffffu, sr, d);
+      si += __shfl_xor_sync(0xffffffffu, si, d);
+    }
+    const int rank = __popc(lanes & ((1u << lane) - 1)), src = 8 * (rank & 3);  // this lane's of the four
+    sr = __shfl_sync(0xffffffffu, sr, src);
+    si = __shfl_sync(0xffffffffu, si, src);
+    if (todo && rank < 4) {
+      double2 v = z[mine * stride];
+      v.x += P.alpha_joined * sr;
+      v.y += P.alpha_joined * si;
+      z[mine * stride] = v;
+      todo &= todo - 1;
+    }
+  }
+}
+
+// Whether a low word of a row's elements k = k0, k0 + step, ... is set.
+__device__ __noinline__ uint32_t low_words(const char* row, const long long* tk, int k0, int step, int klen) {
+  uint32_t any = 0;
+#pragma unroll 1
+  for (int k = k0; k < klen; k += step) {
+    const uint4 v = *reinterpret_cast<const uint4*>(row + tk[k]);
+    any |= v.x | v.z;
+  }
+  return any ? 1u : 0u;
+}
 
 template <int NT, bool AKC, bool BKC>
 __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs P) {
@@ -271,6 +371,10 @@ __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs 
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 6);
   int* sEA = reinterpret_cast<int*>(smem + L::kExpOff);
   long long* sK = reinterpret_cast<long long*>(smem + L::kTabOff);  // k offsets: A, then B
+  uint8_t* sWA = smem + L::kWOff;
+  uint8_t* sWB = sWA + kRows * kWPitch;
+  long long* sAM = reinterpret_cast<long long*>(smem + L::kRowOff);
+  long long* sBN = sAM + kRows;
   long long* sCM = sK + 4 * kSegMax;
   long long* sCN = sCM + kRows;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
@@ -293,7 +397,11 @@ __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs 
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tmem_slot)), "r"(L::kCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  } else if (P.splits == 1) {
+  } else {
+    if (tid < kRows) sAM[tid] = P.aM[min(m0 + tid, P.M - 1)];
+    else if (tid < kRows + NB) sBN[tid - kRows] = P.bN[min(n0 + tid - kRows, P.N - 1)];
+  }
+  if (warp < kWorkers && P.splits == 1) {
     if (tid < kRows) sCM[tid] = m0 + tid < P.M ? P.cM[m0 + tid] : 0;
     else if (tid < kRows + NB) sCN[tid - kRows] = n0 + tid - kRows < P.N ? P.cN[n0 + tid - kRows] : 0;
   }
@@ -375,7 +483,7 @@ __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs 
       const long long* tk = sK + (sg & 1) * 2 * kSegMax;
       int* eA = sEA + (sg & 1) * (kRows + 32);
       int* eB = eA + kRows;
-      if (tid < NB) eB[tid] = kMinExp;
+      if (tid < NB) eB[tid] = kNullRow;
       asm volatile("bar.sync 1, %0;" ::"r"(32 * kWorkers) : "memory");
       auto fetch = [&](int c, double2 (&na)[UA], double2& nb) {
 #pragma unroll
@@ -388,6 +496,13 @@ __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs 
       fetch(1, na1, nb1);
       // ---- exponents of the segment's rows (later stages: read for them only,
       // the conversion finds them in L2 again) ------------------------------------
+      auto word = [](double2 z) {
+        return max(hiabs(uint32_t(__double2hiint(z.x))), hiabs(uint32_t(__double2hiint(z.y))));
+      };
+      // Weight 2^(7 - n) of an element n binades below its row's largest.
+      auto weigh = [&](uint8_t* row, int k, double2 z, int f) {
+        row[k] = uint8_t(__funnelshift_rc(128u, 0u, uint32_t(f - int(word(z) >> 20))));
+      };
       int fa[RA], fb;
       {
         uint32_t ma[RA], mb = 0;
@@ -409,31 +524,51 @@ __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs 
             mb = max(mb, y[c]);
           }
         }
-        auto word = [](double2 z) {
-          return max(hiabs(uint32_t(__double2hiint(z.x))), hiabs(uint32_t(__double2hiint(z.y))));
-        };
 #pragma unroll
         for (int u = 0; u < UA; ++u)
           ma[AKC ? u : 0] = max(ma[AKC ? u : 0], max(word(na0[u]), word(na1[u])));
         mb = max(mb, max(word(nb0), word(nb1)));
+        // the lanes of one row: 16 neighbours (k contiguous) or every eighth lane
+        auto row_max = [](uint32_t v, bool kc) {
+#pragma unroll
+          for (int d = 16; d >= 1; d >>= 1)
+            if (kc ? d < 16 : d >= 8) v = max(v, __shfl_xor_sync(0xffffffffu, v, d));
+          return v;
+        };
+        bool nil = false;
+#pragma unroll
+        for (int u = 0; u < RA; ++u) nil |= (ma[u] = row_max(ma[u], AKC)) == 0;
+        mb = row_max(mb, BKC);
+        if (__any_sync(0xffffffffu, nil || mb == 0)) {
+          // no high word but zeros: zeros, unless a low word says that there
+          // are the smallest of the subnormal numbers
+#pragma unroll
+          for (int u = 0; u < RA; ++u)
+            ma[u] = max(ma[u], row_max(low_words(arow[u], tk, AKC ? lane & 15 : lane >> 3, AKC ? 16 : 4, klen), AKC));
+          mb = max(mb, row_max(low_words(brow, tk + kSegMax, bk(0), kKC, klen), BKC));
+        }
+        auto exponent = [](uint32_t word) {
+          const int f = int(word >> 20);
+          return word == 0 ? kNullRow : (f == 2047 ? kNanExp : max(f, kMinExp));
+        };
 #pragma unroll
         for (int u = 0; u < RA; ++u) {
-          // the lanes of one row: 16 neighbours (AKC) or every eighth lane
-#pragma unroll
-          for (int d = AKC ? 8 : 16; d >= (AKC ? 1 : 8); d >>= 1)
-            ma[u] = max(ma[u], __shfl_xor_sync(0xffffffffu, ma[u], d));
           fa[u] = max(int(ma[u] >> 20), kMinExp);
-          if (AKC ? (lane & 15) == 0 : lane < 8) eA[ar(u)] = fa[u] == 2047 ? kNanExp : fa[u];
+          if (AKC ? (lane & 15) == 0 : lane < 8) eA[ar(u)] = exponent(ma[u]);
         }
 #pragma unroll
-        for (int d = BKC ? 8 : 16; d >= (BKC ? 1 : 8); d >>= 1)
-          mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, d));
-        const int f = int(mb >> 20);
-        if ((BKC ? (lane & 15) == 0 : lane < 8) && br(0) < NB)
-          atomicMax(&eB[br(0)], f == 2047 ? kNanExp : f);
+        for (int u = 0; u < UA; ++u) {
+          weigh(sWA + ar(u) * kWPitch, ak(u), na0[u], fa[AKC ? u : 0]);
+          weigh(sWA + ar(u) * kWPitch, ak(u) + kKC, na1[u], fa[AKC ? u : 0]);
+        }
+        if ((BKC ? (lane & 15) == 0 : lane < 8) && br(0) < NB) atomicMax(&eB[br(0)], exponent(mb));
       }
       asm volatile("bar.sync 1, %0;" ::"r"(32 * kWorkers) : "memory");
-      fb = br(0) < NB ? min(eB[br(0)], 2047) : kMinExp;
+      fb = br(0) < NB ? min(max(eB[br(0)], kMinExp), 2047) : kMinExp;
+      if (br(0) < NB) {
+        weigh(sWB + br(0) * kWPitch, bk(0), nb0, fb);
+        weigh(sWB + br(0) * kWPitch, bk(0) + kKC, nb1, fb);
+      }
       if (sg + 1 < s1) table(sg + 1);
 
       // ---- conversion: elements fetched two stages ahead ----------------------------
@@ -484,6 +619,7 @@ __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs 
       }
 
       // ---- read the accumulators back ---------------------------------------------
+      asm volatile("bar.sync 1, %0;" ::"r"(32 * kWorkers) : "memory");  // sWA, sWB are whole
       if (ok) ok = mbar_wait(smem_u32(done), (sg - s0) & 1, P.budget);
       ok = __all_sync(0xffffffffu, ok);
       const int q = w & 3, c0 = (w >> 2) * CPT;
@@ -500,6 +636,7 @@ __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs 
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const int F = eA[q * 32 + lane] - 2112 + P.ash;
         const uint32_t tq = tmem + (uint32_t(q * 32) << 16) + uint32_t(c0);
+        uint32_t todo = 0;
         // rolled: the code of one tile has to fit the instruction cache
         // (unrolled, fetching it cost more than the work)
 #pragma unroll 1
@@ -509,24 +646,43 @@ __global__ void __launch_bounds__(32 * kWorkers + 32, 1) k_oz_gemm(const OzArgs 
           for (int g = 0; g < kSl; ++g) tmem_ld(tq + uint32_t(g * NT + cc), v[g]);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-          for (int j = 0; j < CU; j += 2) {
+          for (int j = 0; j < CU / 2; ++j) {
+            const int E = F + eB[(c0 + cc) / 2 + j];
             double d[2];
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
               float x[kSl];
 #pragma unroll
-              for (int g = 0; g < kSl; ++g) x[g] = __uint_as_float(v[g][j + i]);
-              d[i] = join(x, F + eB[(c0 + cc + j) >> 1], P.neg);
+              for (int g = 0; g < kSl; ++g) x[g] = __uint_as_float(v[g][2 * j + i]);
+              d[i] = join(x, E, P.neg);
             }
             double2 z = make_double2(d[0], d[1]);
-            if (more) {
-              const double2 o = m < P.M && ((cc + j) >> 1) < ncol ? prow[(long long)((cc + j) >> 1) * P.M] : zero;
-              z.x += o.x; z.y += o.y;
+            const bool in = m < P.M && cc / 2 + j < ncol;
+            const int f = int(max(hiabs(uint32_t(__double2hiint(d[0]))), hiabs(uint32_t(__double2hiint(d[1])))) >> 20);
+            const bool off = f == 2047 || E + kSoundField < 54;
+            if ((off || f < E + kSoundField) && E > kNullRow / 2 && in) {
+              const uint4* wa = reinterpret_cast<const uint4*>(sWA + (q * 32 + lane) * kWPitch);
+              const uint4* wb = reinterpret_cast<const uint4*>(sWB + ((c0 + cc) / 2 + j) * kWPitch);
+              uint32_t sum = 0;
+#pragma unroll
+              for (int u = 0; u < 2; ++u) {
+                const uint4 x = wa[u], y = wb[u];
+                sum = __dp4a(x.x, y.x, __dp4a(x.y, y.y, __dp4a(x.z, y.z, __dp4a(x.w, y.w, sum))));
+              }
+              if (off || sum < kSoundWeight) {
+                todo |= 1u << (cc / 2 + j);
+                z = zero;
+              }
             }
-            if (stage) *reinterpret_cast<double2*>(stg + cc + j) = z;
-            else if (m < P.M && ((cc + j) >> 1) < ncol) prow[(long long)((cc + j) >> 1) * P.M] = z;
+            double2* pz = prow + (long long)(cc / 2 + j) * P.M;
+            if (more && in) { const double2 o = *pz; z.x += o.x; z.y += o.y; }
+            if (stage) *reinterpret_cast<double2*>(stg + cc + 2 * j) = z;
+            else if (in) *pz = z;
           }
         }
+        if (__any_sync(0xffffffffu, todo != 0))
+          settle(P, todo, stage ? reinterpret_cast<double2*>(stg) : prow, stage ? 1 : P.M, sAM + q * 32,
+                 sBN + c0 / 2, tk, klen);
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       }
     }
@@ -717,7 +873,7 @@ int oz_gemm(const OzPlan& p, const OzOperand& A, const OzOperand& B, int M, int 
   a.spc = p.spc;
   a.err = err;
   a.budget = wait_budget > 0 ? wait_budget : kWaitBudget;
-  a.alpha_rest = 1.0;
+  a.alpha_rest = a.alpha_joined = 1.0;
   const bool split = p.nsplit > 1;
   a.splits = p.nsplit;
   a.accumulate = !split && accumulate ? 1 : 0;
@@ -730,6 +886,7 @@ int oz_gemm(const OzPlan& p, const OzOperand& A, const OzOperand& B, int M, int 
     const double f = std::frexp(alpha, &e);
     if (std::fabs(f) == 0.5) {
       a.ash = e - 1;
+      a.alpha_joined = alpha;
       a.neg = alpha < 0 ? 0xffffffffu : 0u;
     } else {
       a.alpha_rest = alpha;

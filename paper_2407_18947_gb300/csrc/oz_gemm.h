@@ -1,17 +1,24 @@
 // FP64-accurate complex products on the tcgen05 tensor cores (sm_103a has 2
 // FP64 FMA lanes per SM and clock; its FP16 tensor pipe does 4096).
 //
-// Error-free splitting (Ozaki, Ogita, Oishi, Rump, "Error-free
+// Splitting (Ozaki, Ogita, Oishi, Rump, "Error-free
 // transformations of matrix multiplication by using fast routines of matrix
 // multiplication and its applications", Numer. Algorithms 59, 95 (2012)):
 // within one K segment every row of A and B is scaled by the power of two
 // above its largest element and rounded to a 62-bit fixed-point number, which
 // is cut into eight balanced 8-bit digits.  The digits are exact in FP16; the
 // 36 digit products i + j <= 7 are formed by FP16 MMAs into eight FP32
-// accumulators (one per i + j) whose partial sums are integers below 2^24 and
-// therefore exact for i + j <= 3 (K <= 256 real; for i + j >= 4, worth at most
-// 2^-46 of the row maxima, a coherent worst case would round once).  The eight
-// sums are joined in integer arithmetic and rounded once to a double.
+// accumulators (one per i + j) whose partial sums are integers up to 2^24 and
+// therefore exact for i + j <= 4 (K <= 256 real; beyond, sums that could have
+// left that range are recognised).  The eight sums are joined in integer
+// arithmetic and rounded once to a double.
+//
+// The error is a fraction of the product of the two rows' largest elements, not
+// of the terms: at most 2 K 8.02 2^-62 of it for K complex terms.  Outputs for
+// which that is not known to be within the bound of FP64 arithmetic, 2 K 2^-53
+// sum |a||b| (opposite gradings, near-identity matrices, infinities and NaN,
+// results below the normal range), are summed in FP64 instead, so that the bound
+// of an FP64 chain holds for every output, |.| being the complex modulus.
 //
 // A complex product C[m,n] (+)= alpha sum_k A[m,k] B[n,k] runs as one real
 // product: A rows interleave (re, im) along K, B is its 2x2 real embedding.
