@@ -1755,7 +1755,9 @@ void Engine<R>::run_contract_small(ContractPlan& P, double alpha, const C* pa, c
                          pc, P.c_off0, kM, kN, Mk, Nk, P.K, P.nsplit, P.kchunk, alpha, accumulate,
                          part, stream_);
   launches_ += P.nsplit > 1 ? 2 : 1;
-  pend(pk, (std::string("contract_small_") + tag).c_str(), 8.0 * mnk, bytes, cur_detail_);
+  pend(pk, (std::string("contract_small_") + tag).c_str(), 8.0 * mnk, bytes,
+       cur_detail_.empty() ? cur_detail_
+                           : "tile=" + std::to_string(int(small_output_tile(P.small_cfg))) + " " + cur_detail_);
 }
 
 template <typename R>
@@ -1814,7 +1816,9 @@ void Engine<R>::run_contract_tc(ContractPlan& P, double alpha, const C* pa, cons
                          (P.tc_nsplit > 1 ? double(P.tc_nsplit) * op.M * 2 * op.N * 4.0
                                           : double(op.M) * op.N * sizeof(C) * (accumulate ? 2.0 : 1.0));
     pend(pk, direct ? "contract_tc_direct_tf32" : (tc_eb_ == 4 ? "contract_tc_tf32" : "contract_tc_bf16"),
-         8.0 * mnk, bytes, cur_detail_);
+         8.0 * mnk, bytes,
+         cur_detail_.empty() || !P.tc_out ? cur_detail_
+                                          : "short=" + std::to_string(P.tc_kp / 32) + " " + cur_detail_);
     ++launches_;
     if (P.tc_nsplit > 1) {
       pk = pbegin();
