@@ -1559,7 +1559,7 @@ ContractPlan& Engine<R>::plan(const std::string& spec, const View& A, const View
   // (a sum of up to six K tiles: its operand's parts fit tensor memory; above
   // 64 complex terms, where the alternative packs both operands too, the line
   // lies where the packed operands are as large as the output)
-  const bool c_unit_m = !gm.empty() && std::llabs(gm.back().sc) == 1;
+  const bool c_unit_m = P->c_unit_m;
   const bool out_bound =
       tc_eb_ == 4 && M * N >= (1LL << 22) && kp_tc <= 64 * kTcShortKb &&
       (long_k ? 2 * M * N >= kp_tc * (c_unit_m ? M + 4 * N : N + 4 * M) : M * N >= 2 * (M + 2 * N) * kp_tc);
