@@ -565,8 +565,14 @@ StageNodes record_stage(Engine<R>& E, const Hamil<R>& H, const StageOptions& opt
   E.axpy(-1.0, t1T, E.v(X).sub(0, o, v).sub(1, 0, o));
   E.axpy(1.0, t1T, E.v(Y).sub(0, o, v).sub(1, 0, o));
   const int LX = E.node({na, n, n}, false, false), Lt = E.node({na, n, n}, false, false);
-  E.contract("pr,Prs->Pps", 1.0, E.v(X), E.v(Lc), E.v(LX), false);
-  E.contract("Pps,sq->Ppq", 1.0, E.v(LX), E.v(Y), E.v(Lt), false);
+  // the identity parts are copies: products with the one block of tau that is not
+  // zero are a fifth of the work, and a near-identity matrix is what the FP64 form's
+  // fixed point holds worst (a tenth of such a product is summed a second time)
+  const View Xt = E.v(X).sub(0, o, v).sub(1, 0, o), Yt = E.v(Y).sub(0, o, v).sub(1, 0, o);
+  E.combine({{1.0, E.v(Lc)}}, E.v(LX), true);
+  E.contract("ai,Pis->Pas", 1.0, Xt, E.v(Lc).sub(1, 0, o), E.v(LX).sub(1, o, v), true);
+  E.combine({{1.0, E.v(LX)}}, E.v(Lt), true);
+  E.contract("Ppa,ai->Ppi", 1.0, E.v(LX).sub(2, o, v), Yt, E.v(Lt).sub(2, 0, o), true);
   const int hw = E.node({n, n}), hX = E.node({n, n}, false, false), ht = E.node({n, n}, false, false);
   E.axpy(1.0, E.v(hc), E.v(hw));
   E.axpy(1.0, E.v(S.w), E.v(hw));
