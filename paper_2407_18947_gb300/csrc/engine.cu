@@ -757,8 +757,9 @@ __global__ void __launch_bounds__(256) k_combine_brick(const BrickDesc<R> d) {
 // Complex128 is bound by the two FP64 FMAs per SM and cycle, not by memory: so
 // there an output skips the sources it has no coefficient for and begins with a
 // term of +-1 at no operation (t, 2t - t - t ...: 10 instead of 24 FMAs per
-// element, (10, 38) 2.78 -> 1.86 ms).  Complex64 is bound by memory (0.50 ms) and
-// keeps the straight sums.
+// element, (10, 38) 2.78 -> 1.86 ms).  Complex64 takes 0.55 ms, 3.2 TB/s of the
+// four tensors it moves (half the copy rate: the permuted reads), and keeps the
+// straight sums.
 enum SumTerm : int { kSumSkip = 0, kSumPlus, kSumMinus, kSumScale, kSumAdd };
 constexpr int kMultiOut = 3;
 template <typename R>
@@ -1429,8 +1430,8 @@ ContractPlan& Engine<R>::plan(const std::string& spec, const View& A, const View
   // FP64 multiply-adds per SM and clock (four per complex one, 85 % of that
   // rate at best, and small outputs are padded to their tile), the sliced form
   // costs what its plan estimates.  Measured, CUDA cores against sliced:
-  // 3800 x 14440 x 48 17.6 -> 1.35 ms, 3800 x 38 x 14440 24.5 -> 1.05 ms, 38 x
-  // 38 x 1.4e6 15.6 -> 3.0 ms, 451 x 451 x 451 0.87 -> 0.054 ms; on the other
+  // 3800 x 14440 x 48 17.6 -> 1.49 ms, 3800 x 38 x 14440 24.5 -> 1.12 ms, 38 x
+  // 38 x 1.4e6 15.6 -> 3.2 ms, 451 x 451 x 451 0.87 -> 0.066 ms; on the other
   // side of the line 10 x 10 x 5.5e6 (4.33 against 4.36 ms) and 144400 x 1 x
   // 380 (0.42 against 0.46 ms) stay on the CUDA cores.
   if (std::is_same<R, double>::value && NB == 1 && K >= 4) {

@@ -17,7 +17,7 @@
 // 85 KB of straight-line code took longer than the work.  Bound by the
 // integer work and load latencies (3800 x 14440 x 48: 52000 warp instructions
 // and 31000 clocks per tile, of which the MMAs take 7000; 17.6 ms on the FP64
-// cores, 1.48 ms here, 0.12 of them for the test that settle() needs).
+// cores, 1.49 ms here, 0.13 of them for the test that settle() needs).
 #include "oz_gemm.h"
 
 #include <cuda_fp16.h>
